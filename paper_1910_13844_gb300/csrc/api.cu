@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <utility>
 #include <vector>
 
 #include "engine.h"
@@ -83,6 +84,86 @@ static int make_twiddles(int L, int R1, int R2, float2** tw, float2** tw2) {
     LS_CUDA_TRY(cudaMalloc(tw2, L * sizeof(float2)));
     LS_CUDA_TRY(cudaMemcpy(*tw2, b.data(), L * sizeof(float2), cudaMemcpyHostToDevice));
   }
+  return LS_OK;
+}
+
+// Launcher, twiddle tables, column order and octant storage of the fused y/z pass, where (ny, nz) has
+// one; a failed allocation leaves the plan with the five passes.
+static int yz_setup(ls_plan* P) {
+  YzLaunch y;
+  switch (P->ny) {
+#define LS_YZ_CASE(N) case N: y = yz_row_##N(P->nz); break;
+    LS_YZ_LENGTHS(LS_YZ_CASE)
+#undef LS_YZ_CASE
+    default: break;
+  }
+  if (!y.run) return LS_OK;
+  const double pi = 3.14159265358979323846;
+  std::vector<float2> yt((size_t)2 * y.ra * y.csp, make_float2(0.f, 0.f)), zt((size_t)y.r1 * y.xr, make_float2(0.f, 0.f));
+  for (int par = 0; par < 2; ++par)
+    for (int c = 0; c < y.ra; ++c)
+      for (int b = 0; b < y.rb; ++b) {
+        const double w = -2.0 * pi * (b * (2 * c + par) % (2 * P->ny)) / (2 * P->ny);
+        yt[((size_t)par * y.ra + c) * y.csp + b] = make_float2((float)cos(w), (float)sin(w));
+      }
+  for (int k1 = 0; k1 < y.r1; ++k1)
+    for (int n2 = 0; n2 < y.r2; ++n2) {
+      const double w = -2.0 * pi * (k1 * n2 % (2 * P->nz)) / (2 * P->nz);
+      zt[(size_t)k1 * y.xr + n2] = make_float2((float)cos(w), (float)sin(w));
+    }
+  // Columns j = c + ra d at tile position c csp + d, in pairs j, j' = -j - P (mod ny): ky and -ky, which share
+  // their Green values (j = 0 and ny / 2 of P = 0 are their own mirrors and make one pair).  The pairs of a
+  // half-warp (16 / tz) are chosen so that their columns lie distinct multiples of tz apart modulo 16
+  // where they can: disjoint banks, as the row pitch is odd.
+  auto entry = [&](int j) { return (j % y.ra * y.csp + j / y.ra) | j << 16; };
+  std::vector<int> cols;
+  for (int par = 0; par < 2; ++par) {
+    std::vector<std::pair<int, int>> left;
+    if (par == 0) left.push_back({entry(0), entry(P->ny / 2)});
+    for (int j = 0; j < P->ny; ++j) {
+      const int m = (2 * P->ny - j - par) % P->ny;
+      if (j < m) left.push_back({entry(j), entry(m)});
+    }
+    const int group = std::max(1, 16 / y.tz);
+    while (!left.empty()) {
+      const std::pair<int, int> first = left.front();
+      unsigned used[2] = {0, 0};
+      for (int h = 0; h < group && !left.empty(); ++h) {
+        size_t k = 0;
+        for (size_t i = 0; i < 2 * left.size(); ++i) {
+          std::pair<int, int> c = left[i / 2];
+          if (i % 2) std::swap(c.first, c.second);
+          const int a = c.first & 0xffff, b = c.second & 0xffff;
+          if ((a - (first.first & 0xffff)) % y.tz == 0 && (b - (first.second & 0xffff)) % y.tz == 0 &&
+              !(used[0] >> (a & 15) & 1u) && !(used[1] >> (b & 15) & 1u)) {
+            k = i / 2;
+            left[k] = c;
+            break;
+          }
+        }
+        used[0] |= 1u << (left[k].first & 15);
+        used[1] |= 1u << (left[k].second & 15);
+        cols.push_back(left[k].first);
+        cols.push_back(left[k].second);
+        left.erase(left.begin() + k);
+      }
+    }
+  }
+  auto upload = [](void** dst, const void* src, size_t bytes) {
+    return cudaMalloc(dst, bytes) == cudaSuccess && cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+  };
+  const bool ok = y.setup() == cudaSuccess &&
+                  cudaMalloc((void**)&P->gyz, (size_t)(P->nx + 1) * (P->ny + 1) * 2 * P->nz * sizeof(float2)) == cudaSuccess &&
+                  upload((void**)&P->yz_ytw, yt.data(), yt.size() * sizeof(float2)) &&
+                  upload((void**)&P->yz_ztw, zt.data(), zt.size() * sizeof(float2)) &&
+                  upload((void**)&P->yz_cols, cols.data(), cols.size() * sizeof(int));
+  if (!ok) {
+    cudaGetLastError();
+    cudaFree(P->gyz);
+    P->gyz = nullptr;
+    return LS_OK;
+  }
+  P->yz = y;
   return LS_OK;
 }
 
@@ -320,12 +401,45 @@ static SlotSel counted(ls_plan* P, SlotSel s, int kind) {
   return s;
 }
 
+// Whether a launch over nslots views runs the fused y/z pass: where (ny, nz) has one, as ls_autotune chose
+// for launches of more than half the tuned batch, else by the pair's measured rule (YZ::large_ok: always,
+// or for launches of at most two waves of its CTAs, where the launches saved count most).  The z pass's
+// waits are under test only in the five-pass form.
+static bool use_fused(const ls_plan* P, int nslots) {
+  if (!P->gyz || P->inj_z_stall || P->inj_z_wait_ns) return false;
+  if (P->tune_fused >= 0 && 2 * nslots > P->tune_views) return P->tune_fused != 0;
+  return P->yz.large_ok || (long long)P->nx * nslots <= (long long)P->sms * P->yz.minb;
+}
+
 static void matvec_core(ls_plan* P, SlotSel sel, int nslots, const FxParams& fx_in, IxParams ix, cudaStream_t st) {
   Engine& e = P->eng;
   FxParams fx = fx_in;
+  const bool fused = use_fused(P, nslots);
   fx.sel = counted(P, fx.sel, LS_K_FX);
   fx.dbg_probe = P->inj_bounds_probe;
+  fx.transposed = ix.transposed = fused ? 1 : 0;
   timed(P, LS_K_FX, nslots, st, [&] { P->px.fx(fx, nslots, st); });
+  ix.sel = counted(P, sel, LS_K_IX);
+  ix.nx = P->nx;
+  ix.rows = P->ny * P->nz;
+  ix.src = e.a1; ix.src_stride = e.a1_stride;
+  ix.tw2 = P->tw2_x;
+  ix.prefetch = P->tune_ix_prefetch;
+  ix.maxparts = e.maxparts;
+  if (fused) {
+    YzParams yz;
+    yz.sel = sel;
+    const int kinds[3] = {LS_K_FY, LS_K_Z, LS_K_IY};
+    for (int i = 0; i < 3; ++i) yz.runs[i] = counted(P, sel, kinds[i]).runs;
+    yz.nx = P->nx;
+    yz.a1 = e.a1; yz.a1_stride = e.a1_stride;
+    yz.g = P->gyz;
+    yz.ytw = P->yz_ytw; yz.ztw = P->yz_ztw; yz.cols = P->yz_cols;
+    yz.sms = P->sms;
+    timed_fused(P, nslots, st, [&] { P->yz.run(yz, nslots, st); });
+    timed(P, LS_K_IX, nslots, st, [&] { P->px.ix(ix, nslots, st); });
+    return;
+  }
   StridedParams fy = fy_base(P, counted(P, sel, LS_K_FY), e.a1, e.a1_stride, e.a2, e.a2_stride, P->nz);
   timed(P, LS_K_FY, nslots, st, [&] { P->py.fy(fy, nslots, st); });
   ZParams z = {};
@@ -359,13 +473,6 @@ static void matvec_core(ls_plan* P, SlotSel sel, int nslots, const FxParams& fx_
   iy.src_plane = (size_t)2 * P->ny * 2 * P->nx;
   iy.dst_plane = (size_t)P->ny * 2 * P->nx;
   timed(P, LS_K_IY, nslots, st, [&] { P->py.iy(iy, nslots, st); });
-  ix.sel = counted(P, sel, LS_K_IX);
-  ix.nx = P->nx;
-  ix.rows = P->ny * P->nz;
-  ix.src = e.a1; ix.src_stride = e.a1_stride;
-  ix.tw2 = P->tw2_x;
-  ix.prefetch = P->tune_ix_prefetch;
-  ix.maxparts = e.maxparts;
   timed(P, LS_K_IX, nslots, st, [&] { P->px.ix(ix, nslots, st); });
 }
 
@@ -559,10 +666,11 @@ void seq_far_adjoint(ls_plan* P, int nslots, const float2* const* r_dev_table, u
 int ensure_iter_graph(ls_plan* P, int nslots) {
   Engine& e = P->eng;
   // the captured launches carry the plan's launch variants: recapture when ls_autotune changed them
-  const int variant = P->tune_z_tma | P->tune_ix_prefetch << 1 | P->tune_fx_views_fastest << 2 |
+  const long long variant = P->tune_z_tma | P->tune_ix_prefetch << 1 | P->tune_fx_views_fastest << 2 |
                       (P->inj_z_stall || P->inj_z_wait_ns ? 1 << 3 : 0) | P->tune_z_split << 4 |
                       P->tune_strided_wide << 5 | (P->tune_z_persist & 3) << 6 | P->tune_fx_bulk << 8 |
-                      (P->tune_views_per_launch & 0x7ff) << 9 | (P->tune_views & 0x7ff) << 20;
+                      (P->tune_views_per_launch & 0x7ff) << 9 | (long long)(P->tune_views & 0x7ff) << 20 |
+                      (long long)((P->tune_fused + 1) & 3) << 31;
   if (e.iter_graph && e.iter_graph_slots == nslots && e.iter_graph_variant == variant) return LS_OK;
   if (e.iter_graph) {
     cudaGraphExecDestroy(e.iter_graph);
@@ -594,6 +702,8 @@ ls_plan plan_slot_view(const ls_plan* P, int s0) {
   v.tune_views = P->tune_views;
   v.gocta = P->gocta; v.k2hat = P->k2hat; v.p_built = P->p_built;
   v.gxz = P->gxz; v.gxz_map = P->gxz_map; v.gxz_ok = P->gxz_ok;
+  v.yz = P->yz; v.gyz = P->gyz; v.yz_ytw = P->yz_ytw; v.yz_ztw = P->yz_ztw; v.yz_cols = P->yz_cols;
+  v.tune_fused = P->tune_fused;
   v.device = P->device; v.sms = P->sms;
   v.tune_z_tma = P->tune_z_tma; v.tune_ix_prefetch = P->tune_ix_prefetch;
   v.tune_fx_views_fastest = P->tune_fx_views_fastest;
@@ -633,6 +743,8 @@ ls_plan* plan_clone_shared(const ls_plan* P) {
   c->tune_views = P->tune_views;
   c->gocta = P->gocta; c->k2hat = P->k2hat; c->p_built = P->p_built;
   c->gxz = P->gxz; c->gxz_map = P->gxz_map; c->gxz_ok = P->gxz_ok;
+  c->yz = P->yz; c->gyz = P->gyz; c->yz_ytw = P->yz_ytw; c->yz_ztw = P->yz_ztw; c->yz_cols = P->yz_cols;
+  c->tune_fused = P->tune_fused;
   c->device = P->device; c->sms = P->sms;
   c->tune_z_tma = P->tune_z_tma; c->tune_ix_prefetch = P->tune_ix_prefetch;
   c->tune_fx_views_fastest = P->tune_fx_views_fastest;
@@ -733,9 +845,18 @@ void prof_resolve(ls_plan* P, bool wait) {
     if (cudaEventQuery(q.b) == cudaSuccess) {
       float ms = 0.f;
       cudaEventElapsedTime(&ms, q.a, q.b);
-      pr.ms[q.kind] += ms;
-      pr.launches[q.kind] += 1;
-      pr.slot_passes[q.kind] += q.slots;
+      if (q.kind == kProfFused) {
+        const int kinds[3] = {LS_K_FY, LS_K_Z, LS_K_IY};
+        for (int k : kinds) {
+          pr.ms[k] += ms * (k == LS_K_Z ? 0.5f : 0.25f);
+          pr.launches[k] += 1;
+          pr.slot_passes[k] += q.slots;
+        }
+      } else {
+        pr.ms[q.kind] += ms;
+        pr.launches[q.kind] += 1;
+        pr.slot_passes[q.kind] += q.slots;
+      }
       pr.pool.push_back(q.a);
       pr.pool.push_back(q.b);
     } else {
@@ -959,6 +1080,7 @@ int ls_plan_create(const ls_grid* grid, int padding, double k_b, double voxel, c
     }
     P->gxz_ok = encode_gxz_map(P) ? 1 : 0;
   }
+  if (rc == LS_OK) rc = yz_setup(P);
   if (rc == LS_OK) rc = ls_green_spectrum(P, P->opt.oversample_p, nullptr, nullptr);
   if (rc == LS_OK) {
     double2* scratch = nullptr;
@@ -994,6 +1116,7 @@ void ls_plan_destroy(ls_plan* P) {
     cudaFree(P->zwa2_z); cudaFree(P->zwb2_z);
     cudaFree(P->twa_z); cudaFree(P->twb_z);
     cudaFree(P->gocta); cudaFree(P->k2hat); cudaFree(P->gxz);
+    cudaFree(P->gyz); cudaFree(P->yz_ytw); cudaFree(P->yz_ztw); cudaFree(P->yz_cols);
   }
   delete P;
 }
@@ -1022,6 +1145,7 @@ int ls_green_spectrum(ls_plan* P, int p, ls_c64* out_full, void* stream) {
     }
     cudaError_t e = build_green_octant(g, S, K, P->gocta, st);
     if (e == cudaSuccess && P->gxz) e = unfold_octant_x(P->nx, P->ny, P->nz, P->gocta, P->gxz, st);
+    if (e == cudaSuccess && P->gyz) e = arrange_octant(P->nx, P->ny, P->nz, P->yz.r1, P->gocta, P->gyz, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(S);
     cudaFree(K);
@@ -1434,7 +1558,11 @@ int ls_debug_bounds(unsigned* site, int clear) {
   unsigned (*const readers[])(bool) = {bounds_site_16,  bounds_site_24,  bounds_site_32,  bounds_site_48,
                                        bounds_site_64,  bounds_site_96,  bounds_site_128, bounds_site_144,
                                        bounds_site_192, bounds_site_256, bounds_site_288, bounds_site_384,
-                                       bounds_site_krylov};
+                                       bounds_site_krylov,
+#define LS_YZ_SITE(N) bounds_site_yz_##N,
+                                       LS_YZ_LENGTHS(LS_YZ_SITE)
+#undef LS_YZ_SITE
+  };
   unsigned first = 0;
   for (auto rd : readers) {
     const unsigned v = rd(clear != 0);

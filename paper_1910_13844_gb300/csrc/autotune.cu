@@ -12,7 +12,8 @@
 //     staged in shared memory, three row blocks ahead) or not, the views per launch of an iteration
 //     (all, or chunks of n/2, n/4 or 8 views, each chunk one launch per pass), iterations between
 //     host reads of the convergence mask (2, 4, 8), and replay of the iteration from a captured CUDA
-//     graph or direct launches.
+//     graph or direct launches;
+//   * the fused y/z pass instead of FY, Z and IY, with the loop variants chosen for those.
 // Operator variants are timed on batched operator applications, the loop variants on forward solves
 // of plane-wave illuminations.  Every operator variant's output is first compared with the default
 // variants' (relative L2 over the batch); a variant that differs by more than 1e-5 is never chosen.
@@ -49,7 +50,7 @@ static std::string tune_key(const ls_plan* P, int n_views) {
   return buf;
 }
 
-static bool cache_lookup(const std::string& key, ls_tune* t) {
+static bool cache_lookup(const std::string& key, ls_tune* t, int* fused) {
   const char* path = getenv("LS_AUTOTUNE_CACHE");
   if (!path || !*path) return false;
   std::lock_guard<std::mutex> lock(g_cache_mu);
@@ -60,11 +61,14 @@ static bool cache_lookup(const std::string& key, ls_tune* t) {
   bool found = false;
   char line[512];
   while (fgets(line, sizeof(line), fp)) {
-    if (sscanf(line, "%255s %d %d %d %d %d %lf %lf %d %d %d %d %d", k, &v.z_tma, &v.ix_prefetch,
+    // an entry without the last field was tuned for the five passes
+    int fu = 0;
+    if (sscanf(line, "%255s %d %d %d %d %d %lf %lf %d %d %d %d %d %d", k, &v.z_tma, &v.ix_prefetch,
                &v.fx_views_fastest, &v.check_every, &v.use_graphs, &v.matvec_us_per_view, &v.solve_ms, &v.z_split,
-               &v.strided_wide, &v.views_per_launch, &v.z_persist, &v.fx_bulk) == 13 &&
+               &v.strided_wide, &v.views_per_launch, &v.z_persist, &v.fx_bulk, &fu) >= 13 &&
         key == k) {
       *t = v;   // the last entry for a key wins
+      *fused = fu != 0;
       found = true;
     }
   }
@@ -72,19 +76,19 @@ static bool cache_lookup(const std::string& key, ls_tune* t) {
   return found;
 }
 
-static void cache_store(const std::string& key, const ls_tune& t) {
+static void cache_store(const std::string& key, const ls_tune& t, int fused) {
   const char* path = getenv("LS_AUTOTUNE_CACHE");
   if (!path || !*path) return;
   std::lock_guard<std::mutex> lock(g_cache_mu);
   FILE* fp = fopen(path, "a");
   if (!fp) return;
-  fprintf(fp, "%s %d %d %d %d %d %.9g %.9g %d %d %d %d %d\n", key.c_str(), t.z_tma, t.ix_prefetch,
+  fprintf(fp, "%s %d %d %d %d %d %.9g %.9g %d %d %d %d %d %d\n", key.c_str(), t.z_tma, t.ix_prefetch,
           t.fx_views_fastest, t.check_every, t.use_graphs, t.matvec_us_per_view, t.solve_ms, t.z_split, t.strided_wide,
-          t.views_per_launch, t.z_persist, t.fx_bulk);
+          t.views_per_launch, t.z_persist, t.fx_bulk, fused);
   fclose(fp);
 }
 
-static void apply(ls_plan* P, const ls_tune& t) {
+static void apply(ls_plan* P, const ls_tune& t, int fused) {
   P->tune_z_tma = t.z_tma;
   P->tune_ix_prefetch = t.ix_prefetch;
   P->tune_fx_views_fastest = t.fx_views_fastest;
@@ -95,6 +99,7 @@ static void apply(ls_plan* P, const ls_tune& t) {
   P->tune_views_per_launch = t.views_per_launch;
   P->tune_z_persist = t.z_persist;
   P->tune_fx_bulk = t.fx_bulk;
+  P->tune_fused = fused;
 }
 
 // mean milliseconds of `reps` calls of fn after one untimed call; negative on error
@@ -131,11 +136,12 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
   int rc = engine_reserve(P, n_views);
   if (rc) return rc;
   ls_tune best;
-  if (cache_lookup(key, &best)) {
+  int fused = 0;   // not part of ls_tune: the plan and the cache file keep it
+  if (cache_lookup(key, &best, &fused)) {
     if (!P->eng.a2_map_ok) best.z_tma = 0;
     if (!P->zwa2_z) best.z_split = 0;
     if (best.views_per_launch >= n_views) best.views_per_launch = 0;
-    apply(P, best);
+    apply(P, best, fused);
     best.from_cache = 1;
     if (out) *out = best;
     return LS_OK;
@@ -176,7 +182,7 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
   cur.from_cache = 0;
   auto matvec = [&] { return tune_matvec(P, f, n_views, st); };
   // reference output of the default variants (y = x - G f x over the batch, kept in the s vectors)
-  apply(P, cur);
+  apply(P, cur, fused);
   if (matvec() != LS_OK) {
     P->prof.on = prof;
     return LS_ECUDA;
@@ -216,14 +222,14 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
     int best_v = *knob;
     for (int i = 0; i < n_values; ++i) {
       *knob = values[i];
-      apply(P, cur);
+      apply(P, cur, fused);
       const double dev = deviation();
       if (!(dev >= 0.0 && dev <= 1e-5)) continue;   // not the same operator: never chosen
       const double ms = time_ms(st, 3, matvec);
       if (ms > 0 && (best_ms < 0 || ms < best_ms)) { best_ms = ms; best_v = values[i]; }
     }
     *knob = best_v;
-    apply(P, cur);
+    apply(P, cur, fused);
     return best_ms;
   };
   static const int two[2] = {1, 0};
@@ -238,6 +244,14 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
   mv_ms = tune_op(&cur.strided_wide, 2, two);
   mv_ms = tune_op(&cur.ix_prefetch, 2, two);
   mv_ms = tune_op(&cur.fx_views_fastest, 2, two);
+  // the fused y/z pass: its operator now (the reference output is still there), its solves below
+  double fused_ms = -1.0;
+  if (P->gyz) {
+    apply(P, cur, 1);
+    const double dev = deviation();
+    if (dev >= 0.0 && dev <= 1e-5) fused_ms = time_ms(st, 3, matvec);
+    apply(P, cur, 0);
+  }
   // solve loop: forward solves of the plane waves
   auto solve = [&] { return tune_forward(P, f, n_views, st); };
   auto solve_views = solve;
@@ -249,13 +263,13 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
     {
       int rcu = engine_reserve_ucache(P, n_views);
       cur.fx_bulk = 0;
-      apply(P, cur);
+      apply(P, cur, fused);
       double best_b_ms = time_ms(st, kSolveReps, solve_views);
       if (rcu == LS_OK)
         LS_CUDA_TRY(cudaMemcpyAsync(e.ucache, e.vptr(V_X), (size_t)n_views * e.N * sizeof(float2),
                                     cudaMemcpyDeviceToDevice, st));
       cur.fx_bulk = 1;
-      apply(P, cur);
+      apply(P, cur, fused);
       const double ms = rcu == LS_OK ? time_ms(st, kSolveReps, solve_views) : -1.0;
       const double dev = ms > 0 ? differ(V_X, e.ucache) : -1.0;
       cur.fx_bulk = (dev >= 0.0 && dev <= 1e-6 && ms > 0 && (best_b_ms < 0 || ms < best_b_ms)) ? 1 : 0;
@@ -271,7 +285,7 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
       for (int cj = 1; cj < ci; ++cj) seen = seen || cands[cj] == cv;
       if (seen) continue;
       cur.views_per_launch = cv;
-      apply(P, cur);
+      apply(P, cur, fused);
       const double ms = time_ms(st, kSolveReps, solve_views);
       if (ms > 0 && (best_c_ms < 0 || ms < best_c_ms)) { best_c_ms = ms; best_c = cv; }
     }
@@ -280,7 +294,7 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
     int best_v = cur.check_every;
     for (int c : chunks) {
       cur.check_every = c;
-      apply(P, cur);
+      apply(P, cur, fused);
       const double ms = time_ms(st, kSolveReps, solve);
       if (ms > 0 && (sv_ms < 0 || ms < sv_ms)) { sv_ms = ms; best_v = c; }
     }
@@ -289,20 +303,30 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
     double best_g_ms = -1.0;
     for (int g : two) {
       cur.use_graphs = g;
-      apply(P, cur);
+      apply(P, cur, fused);
       const double ms = time_ms(st, kSolveReps, solve);
       if (ms > 0 && (best_g_ms < 0 || ms < best_g_ms)) { best_g_ms = ms; best_g = g; }
     }
     cur.use_graphs = best_g;
     if (best_g_ms > 0) sv_ms = best_g_ms;
+    // the fused y/z pass in place of the three (tuned) passes, where the grid has it
+    if (fused_ms > 0) {
+      apply(P, cur, 1);
+      const double ms = time_ms(st, kSolveReps, solve);
+      if (ms > 0 && (sv_ms < 0 || ms < sv_ms)) {
+        fused = 1;
+        mv_ms = fused_ms;
+        sv_ms = ms;
+      }
+    }
   }
-  apply(P, cur);
+  apply(P, cur, fused);
   P->prof.on = prof;
   LS_CUDA_TRY(cudaGetLastError());
   if (mv_ms < 0 || sv_ms < 0) { set_last_error("autotune timing failed"); return LS_ECUDA; }
   cur.matvec_us_per_view = 1e3 * mv_ms / n_views;
   cur.solve_ms = sv_ms;
-  cache_store(key, cur);
+  cache_store(key, cur, fused);
   if (out) *out = cur;
   return LS_OK;
 }

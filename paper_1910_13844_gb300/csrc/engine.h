@@ -10,6 +10,7 @@
 #include "krylov.cuh"
 #include "passes.cuh"
 #include "trace.h"
+#include "yz.cuh"
 
 namespace lsgpu {
 
@@ -40,7 +41,7 @@ struct Engine {
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t iter_graph = nullptr;
   int iter_graph_slots = 0;
-  int iter_graph_variant = 0;   // launch variants the graph was captured with
+  long long iter_graph_variant = 0;   // launch variants the graph was captured with
   float2* vptr(int v, int slot = 0) const { return vec + ((size_t)v * cap + slot) * N; }
 };
 
@@ -73,6 +74,12 @@ struct ls_plan {
   float2* gxz = nullptr;        // the octant unfolded along x (dynamically scheduled z pass), if that pass exists
   CUtensorMap gxz_map;          // TMA map of gxz (valid if gxz_ok)
   int gxz_ok = 0;
+  // fused y/z pass (yz.cuh), where (ny, nz) has one: its launcher, its Green values, its twiddle
+  // tables and column order
+  lsgpu::YzLaunch yz{};
+  float2* gyz = nullptr;
+  float2 *yz_ytw = nullptr, *yz_ztw = nullptr;
+  int* yz_cols = nullptr;
   float2* k2hat = nullptr;
   int p_built = 0;
   bool owns_shared = true;   // false for clones that borrow another plan's spectra and twiddles
@@ -88,6 +95,7 @@ struct ls_plan {
                                   // more than tune_views / 2 views, smaller launches take the ZAuto form
   int tune_fx_bulk = 0;           // bulk-copy-staged persistent first pass
   int tune_strided_wide = 0;      // FY/IY with 32 pencils per CTA (else 16)
+  int tune_fused = -1;            // fused y/z pass: 1 on, 0 off, -1 (untuned) where it exists
   int tune_views_per_launch = 0;  // BiCGStab iteration launched over chunks of this many views (0: all)
   // test-only failure injection (ls_debug_inject); the defaults inject nothing
   int inj_zero_shadow_view = -1;  // this view's shadow residual is zeroed at the start of a solve
@@ -161,5 +169,25 @@ inline void timed(ls_plan* P0, int kind, int nslots, cudaStream_t st, F&& launch
   cudaEventRecord(b, st);
   P->prof.pending.push_back({kind, nslots, a, b});
 }
+
+// The launch of the fused y/z pass: the ranges of the three passes it stands for, nested; the profiler
+// divides its time by their transforms (FY and IY one quarter each, Z a half) and counts it once for each.
+constexpr int kProfFused = LS_K_COUNT;
+template <class F>
+inline void timed_fused(ls_plan* P, int nslots, cudaStream_t st, F&& launch) {
+  TraceRange fy(trace_kind_name(LS_K_FY)), z(trace_kind_name(LS_K_Z));
+  TraceRange iy(trace_kind_name(LS_K_IY));
+  ls_plan* o = prof_owner(P);
+  if (!o->prof.on) {
+    launch();
+    return;
+  }
+  cudaEvent_t a = prof_event(o), b = prof_event(o);
+  cudaEventRecord(a, st);
+  launch();
+  cudaEventRecord(b, st);
+  o->prof.pending.push_back({kProfFused, nslots, a, b});
+}
+
 
 }  // namespace lsgpu

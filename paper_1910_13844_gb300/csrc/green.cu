@@ -148,6 +148,24 @@ __global__ void k_unfold_x(int nx, int ny, int nz, const float2* oct, float2* gx
   }
 }
 
+// Rows of the fused y/z pass (arrange_octant): 32 kx per block, so that the octant is read along kx; a row's
+// entries are written by the block's threads along the row.
+__global__ void k_arrange_octant(int nx1, int ny1, int nz1, int r1, const float2* oct, float2* g) {
+  __shared__ float2 t[32][33];
+  const int L = 2 * (nz1 - 1), ky = blockIdx.z, x0 = blockIdx.x * 32, e0 = blockIdx.y * 32;
+  auto kz_of = [&](int e) {
+    const int k = (e >> 1) % r1 + r1 * (2 * ((e >> 1) / r1) + (e & 1));
+    return k < nz1 ? k : L - k;
+  };
+  for (int i = threadIdx.y; i < 32; i += blockDim.y)
+    if (e0 + i < L && x0 + (int)threadIdx.x < nx1)
+      t[i][threadIdx.x] = oct[((size_t)kz_of(e0 + i) * ny1 + ky) * nx1 + x0 + threadIdx.x];
+  __syncthreads();
+  for (int i = threadIdx.y; i < 32; i += blockDim.y)
+    if (x0 + i < nx1 && e0 + (int)threadIdx.x < L)
+      g[((size_t)(x0 + i) * ny1 + ky) * L + e0 + threadIdx.x] = t[threadIdx.x][i];
+}
+
 // -------------------------------------------------------------- far-field kernels
 // K2[z][dy][dx] = h^3 g(h c(dx), h c(dy), x_gamma - z_c) with g = e^{i k r}/(4 pi r)
 // (eq. def:Green, midpoint rule of eq. Gtild-1); zero at the Nyquist offsets.
@@ -332,6 +350,12 @@ cudaError_t expand_octant(int nx, int ny, int nz, const float2* oct, float2* ful
 cudaError_t unfold_octant_x(int nx, int ny, int nz, const float2* oct, float2* gxz, cudaStream_t st) {
   const size_t total = (size_t)2 * nx * (ny + 1) * (nz + 1);
   k_unfold_x<<<grid_for(total), 256, 0, st>>>(nx, ny, nz, oct, gxz);
+  return cudaGetLastError();
+}
+
+cudaError_t arrange_octant(int nx, int ny, int nz, int r1, const float2* oct, float2* g, cudaStream_t st) {
+  const dim3 grid((nx + 32) / 32, (2 * nz + 31) / 32, ny + 1);
+  k_arrange_octant<<<grid, dim3(32, 8), 0, st>>>(nx + 1, ny + 1, nz + 1, r1, oct, g);
   return cudaGetLastError();
 }
 

@@ -42,6 +42,7 @@ struct FxParams {
   int sms = 0;                 // SMs of the device (grid of the bulk-staged variant)
   int* err = nullptr;          // set to 1 if a wait for a bulk copy gave up (bulk-staged variant)
   int dbg_probe = 0;           // debug build, test only: the plain kernel's slot check excludes the last slot
+  int transposed = 0;          // dst is [2nx][rows] (the fused y/z pass reads it) instead of [rows][2nx]
 };
 
 struct StridedParams {
@@ -94,6 +95,7 @@ struct IxParams {
   int maxparts = 0;            // partial-sum blocks allocated per slot (0: not checked)
   const float2* tw2;
   int prefetch = 0;            // ask L2 for the epilogue operands at kernel start (autotuned)
+  int transposed = 0;          // src is [2nx][rows] (written by the fused y/z pass) instead of [rows][2nx]
 };
 
 // Debug-build index check: element `off` of slot `slot` of a [slots][stride] array whose slots
@@ -187,7 +189,8 @@ struct Geo {
   static constexpr int PS = 16;                              // pencils per CTA, strided passes
   static constexpr int ZMINB = (T * PS > 256) ? 1 : 2;   // resident CTAs per SM asked of the z pass
   static constexpr int SROW = R2 + 1;                        // padded row of the contiguous exchange
-  static constexpr size_t smem_contig = (size_t)PC * R1 * SROW * sizeof(float2);
+  static constexpr int XROW = R1 * SROW | 1;                 // a row's exchange block, odd: PC rows on disjoint banks
+  static constexpr size_t smem_contig = (size_t)PC * XROW * sizeof(float2);
   static constexpr size_t smem_strided = (size_t)L * PS * sizeof(float2);
   static constexpr size_t smem_z = (size_t)(2 * L + L) * PS * sizeof(float2);   // exchange + Ghat + 2 staging halves
 };

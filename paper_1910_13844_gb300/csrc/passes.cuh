@@ -11,6 +11,10 @@
 //   IX  rows (z,y):   IFFT along x, crop x, epilogue            A1             -> [nz][ny][nx]
 // The inverse normalisation 1/(8 nx ny nz) is folded into Ghat.
 //
+// Grids with a fused y/z pass (yz.cuh) run three kernels instead: FX stores A1 transposed
+// (A1t [kx][nz][ny]), the fused pass does FY, Z and IY of one (view, kx) plane on chip, IX reads A1t.
+// Their TR form writes (reads) PC consecutive rows of one kx as one contiguous run.
+//
 // Each length-L transform (L = 2n) is split L = R1 * R2 and done by T = max(R1, R2)
 // threads per pencil in two register stages with one shared-memory exchange:
 //   X[k1 + R1 k2] = sum_n2 W_R2^{n2 k2} W_L^{n2 k1} sum_n1 x[R2 n1 + n2] W_R1^{n1 k1}.
@@ -54,9 +58,37 @@ __device__ __forceinline__ void block_sum_store(const float (&acc)[NV], double* 
   }
 }
 
+// Second stage of the first pass: DFT_R2 of every exchanged row and the store.  Plain form: lanes along
+// kx, [row][2nx].  TR: lanes along the CTA's PC rows, [kx][rows]; the rows of a block are consecutive y
+// (and z) positions, so PC lanes write one contiguous run.  The odd pitch of a row's exchange block keeps
+// both directions free of bank conflicts.
+template <int L, bool TR>
+__device__ __forceinline__ void fx_store(const FxParams& a, const float2* sm, int slot, int rb) {
+  using G = Geo<L>;
+  constexpr int R1 = G::R1, R2 = G::R2, PC = G::PC;
+  const int tid = threadIdx.y * G::T + threadIdx.x;
+  const int p = TR ? tid % PC : threadIdx.y, t = TR ? tid / PC : threadIdx.x;
+  const int row = rb * PC + p;
+  if (row >= a.rows || t >= R1) return;
+  const float2* S = sm + (size_t)p * G::XROW + t * G::SROW;
+  float2 u[R2];
+#pragma unroll
+  for (int n2 = 0; n2 < R2; ++n2) u[n2] = S[n2];
+  Dft<R2, -1>::run(u);
+  float2* d = a.dst + (size_t)slot * a.dst_stride + (TR ? (size_t)row : (size_t)row * L);
+#pragma unroll
+  for (int k2 = 0; k2 < R2; ++k2) {
+    const int kx = t + R1 * k2;
+    const size_t o = TR ? (size_t)kx * a.rows : (size_t)kx;
+    if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, o + (TR ? (size_t)row : (size_t)row * L), (size_t)a.rows * L,
+                                  a.dst_stride), BS_FX_DST))
+      d[o] = u[k2];
+  }
+}
+
 // ------------------------------------------------------------------------- FX
-template <int L>
-__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 6) k_fx(FxParams a) {
+template <int L, bool TR>
+__device__ __forceinline__ void fx_body(const FxParams& a) {
   using G = Geo<L>;
   constexpr int R1 = G::R1, R2 = G::R2;
   extern __shared__ float2 sm[];
@@ -117,7 +149,7 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 6) k_fx(FxParams a) {
       v[n1] = val;
     }
   }
-  float2* S = sm + (size_t)p * R1 * G::SROW;
+  float2* S = sm + (size_t)p * G::XROW;
   if (t < R2) {
     Dft<R1, -1, R1 / 2, R1>::run(v);
 #pragma unroll
@@ -126,19 +158,13 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 6) k_fx(FxParams a) {
     for (int k1 = 0; k1 < R1; ++k1) S[k1 * G::SROW + t] = v[k1];
   }
   __syncthreads();
-  if (valid && t < R1) {
-    float2 u[R2];
-#pragma unroll
-    for (int n2 = 0; n2 < R2; ++n2) u[n2] = S[t * G::SROW + n2];
-    Dft<R2, -1>::run(u);
-    float2* d = a.dst + (size_t)slot * a.dst_stride + (size_t)row * L;
-#pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2)
-      if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)row * L + t + R1 * k2, (size_t)a.rows * L,
-                                    a.dst_stride), BS_FX_DST))
-        d[t + R1 * k2] = u[k2];
-  }
+  fx_store<L, TR>(a, sm, slot, rb);
 }
+
+template <int L>
+__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 6) k_fx(FxParams a) { fx_body<L, false>(a); }
+template <int L>
+__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 6) k_fx_t(FxParams a) { fx_body<L, true>(a); }
 
 // ------------------------------------------------------------------------- FX (bulk-copy staged)
 // The same pass with the rows of every input vector staged in shared memory by bulk copies
@@ -166,8 +192,8 @@ struct FXB {
   static constexpr bool ok = smem <= 227 * 1024 && stage_bytes % 16 == 0 && vec_bytes % 16 == 0;
 };
 
-template <int L>
-__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 1) k_fxb(FxParams a) {
+template <int L, bool TR>
+__device__ __forceinline__ void fxb_body(const FxParams& a) {
   using G = Geo<L>;
   using B = FXB<L>;
   constexpr int R1 = G::R1, R2 = G::R2, PC = G::PC, NX = B::NX, NSTG = B::NSTG;
@@ -287,7 +313,7 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 1) k_fxb(FxParams a) {
         v[n1] = val;
       }
     }
-    float2* S = S0 + (size_t)p * R1 * G::SROW;
+    float2* S = S0 + (size_t)p * G::XROW;
     if (t < R2) {
       Dft<R1, -1, R1 / 2, R1>::run(v);
 #pragma unroll
@@ -298,22 +324,16 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 1) k_fxb(FxParams a) {
     __syncthreads();
     // every thread has read its inputs from stage s: refill it with the item NSTG ahead
     if (tid == 0 && m + NSTG < nmine) issue(m + NSTG, s);
-    if (valid && t < R1) {
-      float2 u[R2];
-#pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) u[n2] = S[t * G::SROW + n2];
-      Dft<R2, -1>::run(u);
-      float2* d = a.dst + (size_t)slot * a.dst_stride + (size_t)row * L;
-#pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2)
-        if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)row * L + t + R1 * k2, (size_t)a.rows * L,
-                                      a.dst_stride), BS_FX_DST))
-          d[t + R1 * k2] = u[k2];
-    }
+    fx_store<L, TR>(a, S0, slot, rb);
     __syncthreads();   // the exchange area is free for the next item
   }
   (void)NT;
 }
+
+template <int L>
+__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 1) k_fxb(FxParams a) { fxb_body<L, false>(a); }
+template <int L>
+__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 1) k_fxb_t(FxParams a) { fxb_body<L, true>(a); }
 
 // ------------------------------------------------------------------------- FY / IY
 // Pencils along a strided axis; tile = 16 consecutive entries of the contiguous axis.
@@ -404,10 +424,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p));
 }
 
-// Five resident CTAs of 256 threads, six of 192 (24 or 12 threads per row): IX at 192^3 ran at 5.07
-// TB/s with five and 5.70 with six, at 144^3 4.32 and 4.89; at 128^3 six cost 15%.
-template <int L>
-__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, Geo<L>::T * Geo<L>::PC <= 192 ? 6 : 5) k_ix(IxParams a) {
+template <int L, bool TR>
+__device__ __forceinline__ void ix_body(const IxParams& a) {
   using G = Geo<L>;
   constexpr int R1 = G::R1, R2 = G::R2;
   extern __shared__ float2 sm[];
@@ -427,26 +445,33 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, Geo<L>::T * Geo<L>::PC
     if (t < lines) prefetch_l2(a.in0 + voff0 + 16 * t);
     else if (t < 2 * lines && (a.mode == IX_BICG_V || a.mode == IX_RESID)) prefetch_l2(a.in1 + voff0 + 16 * (t - lines));
   }
+  // first stage: TR takes the CTA's rows along the lanes (see fx_store)
+  const int tid = p * G::T + t;
+  const int p1 = TR ? tid % G::PC : p, t1 = TR ? tid / G::PC : t;
+  const int row1 = blockIdx.x * G::PC + p1;
   float2 v[R1];
 #pragma unroll
   for (int n1 = 0; n1 < R1; ++n1) v[n1] = make_float2(0.f, 0.f);
-  if (valid && t < R2) {
-    const float2* s = a.src + (size_t)slot * a.src_stride + (size_t)row * L;
+  if (row1 < a.rows && t1 < R2) {
+    const float2* s = a.src + (size_t)slot * a.src_stride + (TR ? (size_t)row1 : (size_t)row1 * L);
 #pragma unroll
-    for (int n1 = 0; n1 < R1; ++n1)
-      if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)row * L + R2 * n1 + t, (size_t)a.rows * L,
+    for (int n1 = 0; n1 < R1; ++n1) {
+      const size_t o = TR ? (size_t)(R2 * n1 + t1) * a.rows : (size_t)(R2 * n1 + t1);
+      if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, o + (TR ? (size_t)row1 : (size_t)row1 * L), (size_t)a.rows * L,
                                     a.src_stride), BS_IX_SRC))
-        v[n1] = __ldg(s + R2 * n1 + t);
+        v[n1] = __ldg(s + o);
+    }
   }
-  float2* S = sm + (size_t)p * R1 * G::SROW;
-  if (t < R2) {
+  if (t1 < R2) {
+    float2* S1 = sm + (size_t)p1 * G::XROW;
     Dft<R1, +1>::run(v);
 #pragma unroll
-    for (int k1 = 1; k1 < R1; ++k1) v[k1] = cmulc(v[k1], __ldg(a.tw2 + k1 * R2 + t));
+    for (int k1 = 1; k1 < R1; ++k1) v[k1] = cmulc(v[k1], __ldg(a.tw2 + k1 * R2 + t1));
 #pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) S[k1 * G::SROW + t] = v[k1];
+    for (int k1 = 0; k1 < R1; ++k1) S1[k1 * G::SROW + t1] = v[k1];
   }
   __syncthreads();
+  const float2* S = sm + (size_t)p * G::XROW;
   float acc[3] = {0.f, 0.f, 0.f};
   if (valid && t < R1) {
     float2 u[R2];
@@ -505,6 +530,14 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, Geo<L>::T * Geo<L>::PC
   }
 }
 
+// Five resident CTAs of 256 threads, six of 192 (24 or 12 threads per row): IX at 192^3 ran at 5.07
+// TB/s with five and 5.70 with six, at 144^3 4.32 and 4.89; at 128^3 six cost 15%.
+template <int L> struct IxCtas { static constexpr int MINB = Geo<L>::T * Geo<L>::PC <= 192 ? 6 : 5; };
+template <int L>
+__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, IxCtas<L>::MINB) k_ix(IxParams a) { ix_body<L, false>(a); }
+template <int L>
+__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, IxCtas<L>::MINB) k_ix_t(IxParams a) { ix_body<L, true>(a); }
+
 // ------------------------------------------------------------------------- launchers
 struct PassLaunch {
   void (*fx)(const FxParams&, int nslots, cudaStream_t);
@@ -535,7 +568,9 @@ struct PassImpl {
         const int nrb = (a.rows + G::PC - 1) / G::PC;
         FxParams b = a;
         b.sel.nslots = nslots;   // the kernel builds its list of active views from the selector
-        k_fxb<L><<<std::min(nrb * nslots, a.sms), dim3(G::T, G::PC), FXB<L>::smem, st>>>(b);
+        const int grid = std::min(nrb * nslots, a.sms);
+        if (a.transposed) k_fxb_t<L><<<grid, dim3(G::T, G::PC), FXB<L>::smem, st>>>(b);
+        else k_fxb<L><<<grid, dim3(G::T, G::PC), FXB<L>::smem, st>>>(b);
         return;
       }
     }
@@ -543,13 +578,15 @@ struct PassImpl {
     dim3 blk(G::T, G::PC), grd = a.views_fastest ? dim3(nslots, rbs) : dim3(rbs, nslots);
     FxParams b = a;
     b.sel.nslots = nslots;
-    k_fx<L><<<grd, blk, G::smem_contig, st>>>(b);
+    if (a.transposed) k_fx_t<L><<<grd, blk, G::smem_contig, st>>>(b);
+    else k_fx<L><<<grd, blk, G::smem_contig, st>>>(b);
   }
   static void ix(const IxParams& a0, int nslots, cudaStream_t st) {
     IxParams a = a0;
     a.sel.nslots = nslots;
     dim3 blk(G::T, G::PC), grd((a.rows + G::PC - 1) / G::PC, nslots);
-    k_ix<L><<<grd, blk, G::smem_contig, st>>>(a);
+    if (a.transposed) k_ix_t<L><<<grd, blk, G::smem_contig, st>>>(a);
+    else k_ix<L><<<grd, blk, G::smem_contig, st>>>(a);
   }
   template <int DIR>
   static void strided(const StridedParams& a0, int nslots, cudaStream_t st) {
@@ -640,10 +677,17 @@ struct PassImpl {
   static cudaError_t setup() {
     cudaError_t e = cudaSuccess;
     {
-      e = cudaFuncSetAttribute(k_fx<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem_contig);
-      if constexpr (FXB<L>::ok)
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fxb<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FXB<L>::smem);
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ix<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem_contig);
+      auto room = [&](auto kernel, size_t bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+      };
+      room(k_fx<L>, G::smem_contig);
+      room(k_fx_t<L>, G::smem_contig);
+      if constexpr (FXB<L>::ok) {
+        room(k_fxb<L>, FXB<L>::smem);
+        room(k_fxb_t<L>, FXB<L>::smem);
+      }
+      room(k_ix<L>, G::smem_contig);
+      room(k_ix_t<L>, G::smem_contig);
       if (e == cudaSuccess) e = set_strided_smem<-1, G::PS>((int)G::smem_strided);
       if (e == cudaSuccess) e = set_strided_smem<+1, G::PS>((int)G::smem_strided);
       if constexpr (G::T * 32 <= 1024) {
