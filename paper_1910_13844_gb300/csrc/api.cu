@@ -167,9 +167,13 @@ static int yz_setup(ls_plan* P) {
   return LS_OK;
 }
 
-void slot_defaults(const ls_plan* P, SlotDev& s, const float* f, int adjoint) {
+void slot_defaults(const ls_plan* P, SlotDev& s, int slot, const float* f, int adjoint) {
   memset(&s, 0, sizeof(s));
   s.f = f;
+  const Engine& e = P->eng;
+  s.b = s.bo = e.vptr(V_B, slot);
+  s.x = s.xo = e.vptr(V_X, slot);
+  s.far = e.far + (size_t)slot * P->mx * P->my;
   s.flags = SLOT_RESID;
   s.adjoint = adjoint;
   s.first = 1;
@@ -493,13 +497,10 @@ void seq_resid(ls_plan* P, int nslots, cudaStream_t st) {
   Engine& e = P->eng;
   SlotSel sel = sel_slots(P, SLOT_RESID);
   FxParams fx = fx_base(P, sel, P->ny * P->nz);
-  fx.mode = FX_F_TIMES;
-  fx.src = e.vptr(V_X);
+  fx.mode = FX_F_TIMES;   // of the slots' fields x
   IxParams ix;
   memset(&ix, 0, sizeof(ix));
-  ix.mode = IX_RESID;
-  ix.in0 = e.vptr(V_X);
-  ix.in1 = e.vptr(V_B);
+  ix.mode = IX_RESID;     // the slots' x and b
   ix.out0 = e.vptr(V_R);
   ix.out1 = e.vptr(V_RH);
   ix.vstride = e.N;
@@ -557,7 +558,7 @@ void seq_iter(ls_plan* P, int nslots, cudaStream_t st) {
     u.sel = counted(P, sel, LS_K_UPDATE);
     u.n = e.N;
     u.vstride = e.N;
-    u.x = e.vptr(V_X); u.r = e.vptr(V_R);
+    u.r = e.vptr(V_R);
     u.p = e.vptr(V_P); u.s = e.vptr(V_S); u.t = e.vptr(V_T); u.rh = e.vptr(V_RH);
     u.partials = e.partials;
     u.maxparts = e.maxparts;
@@ -580,13 +581,12 @@ void seq_iter_chunked(ls_plan* P, int nslots, cudaStream_t st) {
   }
 }
 
-// far[s] = G~ (f x_s) for the selected slots (eq. Gtild-1)
+// G~ (f x_s) for the selected slots, into their far buffers (eq. Gtild-1)
 void seq_far(ls_plan* P, int nslots, unsigned mask, cudaStream_t st) {
   Engine& e = P->eng;
   SlotSel sel = sel_slots(P, mask);
   FxParams fx = fx_base(P, sel, P->ny * P->nz);
-  fx.mode = FX_F_TIMES;
-  fx.src = e.vptr(V_X);
+  fx.mode = FX_F_TIMES;   // of the slots' fields x
   timed(P, LS_K_FX, nslots, st, [&] { P->px.fx(fx, nslots, st); });
   StridedParams fy = fy_base(P, sel, e.a1, e.a1_stride, e.a2, e.a2_stride, P->nz);
   timed(P, LS_K_FY, nslots, st, [&] { P->py.fy(fy, nslots, st); });
@@ -610,14 +610,14 @@ void seq_far(ls_plan* P, int nslots, unsigned mask, cudaStream_t st) {
   ix.nx = P->nx;
   ix.rows = P->my;
   ix.src = e.a2; ix.src_stride = e.a2_stride;
-  ix.out0 = e.far;
+  ix.out_slot = IX_OUT_FAR;
   ix.vstride = (size_t)P->mx * P->my;
   ix.out_o = P->ox; ix.out_m = P->mx;
   ix.tw2 = P->tw2_x;
   timed(P, LS_K_FAR, nslots, st, [&] { P->px.ix(ix, nslots, st); });
 }
 
-// b_s = G~^H r_s for the selected slots; r_dev_table holds one device pointer per slot
+// G~^H r_s for the selected slots, into their bo vectors; r_dev_table holds one device pointer per slot
 void seq_far_adjoint(ls_plan* P, int nslots, const float2* const* r_dev_table, unsigned mask, cudaStream_t st) {
   Engine& e = P->eng;
   SlotSel sel = sel_slots(P, mask);
@@ -655,7 +655,7 @@ void seq_far_adjoint(ls_plan* P, int nslots, const float2* const* r_dev_table, u
   ix.nx = P->nx;
   ix.rows = P->ny * P->nz;
   ix.src = e.a1; ix.src_stride = e.a1_stride;
-  ix.out0 = e.vptr(V_B);
+  ix.out_slot = IX_OUT_BO;
   ix.vstride = e.N;
   ix.out_o = 0; ix.out_m = P->nx;
   ix.tw2 = P->tw2_x;
@@ -755,7 +755,7 @@ ls_plan* plan_clone_shared(const ls_plan* P) {
 int tune_matvec(ls_plan* P, const float* f, int n, cudaStream_t st) {
   Engine& e = P->eng;
   for (int q = 0; q < n; ++q) {
-    slot_defaults(P, e.slots_h[q], f, 0);
+    slot_defaults(P, e.slots_h[q], q, f, 0);
     e.slots_h[q].flags = SLOT_AUX;
   }
   LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, e.slots_h, (size_t)n * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
@@ -778,7 +778,7 @@ int tune_forward(ls_plan* P, const float* f, int n, cudaStream_t st) {
   Engine& e = P->eng;
   LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X), e.vptr(V_B), (size_t)n * e.N * sizeof(float2), cudaMemcpyDeviceToDevice,
                               st));
-  for (int q = 0; q < n; ++q) slot_defaults(P, e.slots_h[q], f, 0);
+  for (int q = 0; q < n; ++q) slot_defaults(P, e.slots_h[q], q, f, 0);
   return engine_solve(P, n, st);
 }
 
@@ -794,34 +794,46 @@ int engine_solve(ls_plan* P, int nslots, cudaStream_t st) {
     if (rc != LS_OK) return rc;
   }
   const int chunk = P->opt.check_every > 0 ? P->opt.check_every : 2;
-  long long max_rounds = (long long)P->opt.max_iter * (P->opt.max_restarts + 2) / chunk + 16;
-  if (P->inj_max_rounds >= 0) max_rounds = std::min(max_rounds, P->inj_max_rounds);
-  for (long long round = 0; round < max_rounds; ++round) {
-    timed(P, LS_K_OTHER, nslots, st, [&] { launch_count(e.slots_d, nslots, e.counts_d, st); });
-    LS_CUDA_TRY(cudaMemcpyAsync(e.counts_h, e.counts_d, 5 * sizeof(int), cudaMemcpyDeviceToHost, st));
+  // Rounds: a residual evaluation or a chunk of iterations.  The iterations that follow the initial
+  // residual need no look at the states in between (views that start converged are masked off), so the
+  // two go out together.
+  long long left = (long long)P->opt.max_iter * (P->opt.max_restarts + 2) / chunk + 16;
+  if (P->inj_max_rounds >= 0) left = std::min(left, P->inj_max_rounds);
+  int n_iter = 0, n_resid = nslots;
+  bool first = true;
+  if (left <= 0) LS_CUDA_TRY(cudaStreamSynchronize(st));   // slots_h is uploaded when this returns
+  while (left > 0 && (n_iter > 0 || n_resid > 0)) {
+    if (n_resid > 0) {
+      seq_resid(P, nslots, st);
+      --left;
+    }
+    if (left > 0 && (n_iter > 0 || first)) {
+      for (int k = 0; k < chunk; ++k) {
+        if (graphs) {
+          LS_CUDA_TRY(cudaGraphLaunch(e.iter_graph, st));
+        } else {
+          seq_iter_chunked(P, nslots, st);
+        }
+      }
+      --left;
+    }
+    first = false;
+    LS_CUDA_TRY(cudaGetLastError());
+    // the states and the error word come back together
+    LS_CUDA_TRY(cudaMemcpyAsync(e.slots_h, e.slots_d, (size_t)nslots * sizeof(SlotDev), cudaMemcpyDeviceToHost, st));
+    LS_CUDA_TRY(cudaMemcpyAsync(e.counts_h + 4, e.counts_d + 4, sizeof(int), cudaMemcpyDeviceToHost, st));
     LS_CUDA_TRY(cudaStreamSynchronize(st));
     prof_resolve(P, false);
     if (e.counts_h[4]) {
       set_last_error("a TMA copy of the z pass or a bulk copy of the first pass did not complete within its time limit");
       return LS_ECUDA;
     }
-    const int n_iter = e.counts_h[0], n_resid = e.counts_h[1];
-    if (n_iter == 0 && n_resid == 0) break;
-    if (n_resid > 0) {
-      seq_resid(P, nslots, st);
-      continue;
+    n_iter = n_resid = 0;
+    for (int q = 0; q < nslots; ++q) {
+      n_iter += (e.slots_h[q].flags & SLOT_ITER) ? 1 : 0;
+      n_resid += (e.slots_h[q].flags & SLOT_RESID) ? 1 : 0;
     }
-    for (int k = 0; k < chunk; ++k) {
-      if (graphs) {
-        LS_CUDA_TRY(cudaGraphLaunch(e.iter_graph, st));
-      } else {
-        seq_iter_chunked(P, nslots, st);
-      }
-    }
-    LS_CUDA_TRY(cudaGetLastError());
   }
-  LS_CUDA_TRY(cudaMemcpyAsync(e.slots_h, e.slots_d, (size_t)nslots * sizeof(SlotDev), cudaMemcpyDeviceToHost, st));
-  LS_CUDA_TRY(cudaStreamSynchronize(st));
   return LS_OK;
 }
 
@@ -898,6 +910,29 @@ static int pupil_adjoint_residuals(ls_plan* P, int n, const ls_c64* const* r, st
   LS_CUDA_TRY(cudaFreeAsync(scratch, st));
   return rc;
 }
+
+static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+// Caller memory that a batched call reads or writes while it runs.
+struct Spans {
+  struct Span { uintptr_t a, b; bool w; };
+  std::vector<Span> v;
+  void add(const void* p, size_t bytes, bool written) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    v.push_back({a, a + bytes, written});
+  }
+  // no written range overlaps another range
+  bool disjoint() {
+    std::sort(v.begin(), v.end(), [](const Span& x, const Span& y) { return x.a < y.a; });
+    uintptr_t any = 0, written = 0;
+    for (const Span& s : v) {
+      if (s.a < (s.w ? any : written)) return false;
+      any = std::max(any, s.b);
+      if (s.w) written = std::max(written, s.b);
+    }
+    return true;
+  }
+};
 
 static int worst_status(const Engine& e, int nslots, ls_stats* stats) {
   int worst = LS_OK;
@@ -1240,25 +1275,40 @@ int ls_matvec_batch(ls_plan* P, const float* f, int n_views, const ls_c64* const
   rc = engine_reserve(P, n_views);
   if (rc) return rc;
   Engine& e = P->eng;
+  // The passes read x[q] and write y[q] where they are; in place (y[q] == x[q]) each element is read by
+  // the thread that writes it.  Where an output overlaps another vector the call works on copies.
+  Spans io;
   for (int q = 0; q < n_views; ++q) {
-    LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), x[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
-    slot_defaults(P, e.slots_h[q], f, adjoint ? 1 : 0);
-    e.slots_h[q].flags = SLOT_AUX;
+    io.add(y[q], e.N * sizeof(float2), true);
+    if (x[q] != y[q]) io.add(x[q], e.N * sizeof(float2), false);
   }
-  LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, e.slots_h, (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
+  const bool direct = io.disjoint();
+  // states from pageable memory: the copy is taken before the call returns (the call does not synchronise)
+  std::vector<SlotDev> slots(n_views);
+  for (int q = 0; q < n_views; ++q) {
+    slot_defaults(P, slots[q], q, f, adjoint ? 1 : 0);
+    slots[q].flags = SLOT_AUX;
+    slots[q].xo = e.vptr(V_R, q);
+    if (direct) {
+      slots[q].x = (const float2*)x[q];
+      slots[q].xo = (float2*)y[q];
+    } else {
+      LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), x[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+    }
+  }
+  LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, slots.data(), (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
   SlotSel sel = sel_slots(P, SLOT_AUX);
   FxParams fx = fx_base(P, sel, P->ny * P->nz);
   fx.mode = FX_F_TIMES;
-  fx.src = e.vptr(V_X);
   IxParams ix;
   memset(&ix, 0, sizeof(ix));
   ix.mode = IX_MATVEC;
-  ix.in0 = e.vptr(V_X);
-  ix.out0 = e.vptr(V_R);
+  ix.out_slot = IX_OUT_XO;
   ix.vstride = e.N;
   matvec_core(P, sel, n_views, fx, ix, st);
-  for (int q = 0; q < n_views; ++q)
-    LS_CUDA_TRY(cudaMemcpyAsync(y[q], e.vptr(V_R, q), e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+  if (!direct)
+    for (int q = 0; q < n_views; ++q)
+      LS_CUDA_TRY(cudaMemcpyAsync(y[q], e.vptr(V_R, q), e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
   LS_CUDA_TRY(cudaGetLastError());
   prof_resolve(P, false);
   return LS_OK;
@@ -1277,44 +1327,55 @@ static void builtin_kvec(const ls_plan* P, int n, std::vector<double>& k) {
   }
 }
 
-// Built-in plane waves for slots [0, n), written straight into b and (unless initial guesses are
-// given) x0 = b: one launch over a pointer table of 2n (or n) vectors.
-static int builtin_plane_waves(ls_plan* P, int n, bool also_x, cudaStream_t st) {
+// Built-in plane waves for slots [0, n), written straight into the b vectors.
+static int builtin_plane_waves(ls_plan* P, int n, cudaStream_t st) {
   Engine& e = P->eng;
   std::vector<double> k;
   builtin_kvec(P, n, k);
-  const int m = also_x ? 2 * n : n;
-  if (also_x) k.insert(k.end(), k.begin(), k.end());
-  std::vector<void*> ptrs(m);
-  for (int q = 0; q < n; ++q) {
-    ptrs[q] = e.vptr(V_B, q);
-    if (also_x) ptrs[n + q] = e.vptr(V_X, q);
-  }
-  // the kvec table holds 6 * cap doubles and the pointer tables 4 * cap pointers: tables 0 and 1 carry 2n
+  std::vector<void*> ptrs(n);
+  for (int q = 0; q < n; ++q) ptrs[q] = e.vptr(V_B, q);
   LS_CUDA_TRY(cudaMemcpyAsync(e.kvec_d, k.data(), k.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-  int rc = engine_upload_ptrs(P, 0, (const void* const*)ptrs.data(), m, st);
+  int rc = engine_upload_ptrs(P, 0, (const void* const*)ptrs.data(), n, st);
   if (rc) return rc;
   PlaneWaveParams a{P->nx, P->ny, P->nz, P->h, e.kvec_d, (float2* const*)engine_ptr_table(P, 0)};
-  LS_CUDA_TRY(launch_plane_waves(a, m, st));
+  LS_CUDA_TRY(launch_plane_waves(a, n, st));
   return LS_OK;
 }
 
-// Copy the caller's right-hand sides into slots [0, n) (b, and x0 = b unless initial guesses are given)
-// and set the slot states.  rhs == NULL: the plan's built-in plane waves.
-static int load_rhs(ls_plan* P, const float* f, int n, const ls_c64* const* rhs, int adjoint, cudaStream_t st,
-                    const ls_c64* const* x0 = nullptr) {
+// Slot states of a solve of n views with right-hand sides rhs (NULL: the plan's built-in plane waves) and
+// initial guesses x0 (NULL: the right-hand sides).  The solve reads the caller's right-hand sides and
+// guesses where they are and updates the fields in out[q] (NULL: in the workspace), unless `copy` (an
+// output overlaps another of the call's vectors): then it works on copies in the workspace.  Fields are
+// read and written 16 bytes at a time by the update, so a pointer that is not so aligned takes the
+// workspace too.
+static int load_rhs(ls_plan* P, const float* f, int n, const ls_c64* const* rhs, const ls_c64* const* x0, bool copy,
+                    float2* const* out, cudaStream_t st) {
   Engine& e = P->eng;
   if (!rhs) {
-    int rc = builtin_plane_waves(P, n, x0 == nullptr, st);
+    int rc = builtin_plane_waves(P, n, st);
     if (rc) return rc;
   }
   for (int q = 0; q < n; ++q) {
-    if (rhs) LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_B, q), rhs[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
-    if (rhs || x0)
-      LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), x0 ? x0[q] : rhs[q], e.N * sizeof(float2),
-                                  cudaMemcpyDeviceToDevice, st));
+    SlotDev& s = e.slots_h[q];
+    slot_defaults(P, s, q, f, 0);
+    if (rhs && copy)
+      LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_B, q), rhs[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+    else if (rhs)
+      s.b = (const float2*)rhs[q];
+    const float2* x = x0 ? (const float2*)x0[q] : s.b;
+    if ((x0 && copy) || !aligned16(x))
+      LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), x, e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+    else
+      s.x = x;
+    if (!copy && out && out[q] && aligned16(out[q])) s.xo = out[q];
   }
-  for (int q = 0; q < n; ++q) slot_defaults(P, e.slots_h[q], f, adjoint);
+  return LS_OK;
+}
+
+// out[q] <- the slot's field, unless the solve left it there
+static int store_field(const Engine& e, int q, void* out, cudaStream_t st) {
+  if (e.slots_h[q].x != out)
+    LS_CUDA_TRY(cudaMemcpyAsync(out, e.slots_h[q].x, e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
   return LS_OK;
 }
 
@@ -1331,8 +1392,21 @@ static int forward_impl(ls_plan* P, const float* f, int n_views, const ls_c64* c
   rc = engine_reserve(P, n_views);
   if (rc) return rc;
   Engine& e = P->eng;
-  rc = load_rhs(P, f, n_views, u_in, 0, st, x0);
+  const size_t fb = e.N * sizeof(float2), db = (size_t)P->mx * P->my * sizeof(float2);
+  Spans io;
+  io.add(f, e.N * sizeof(float), false);
+  for (int q = 0; q < n_views; ++q) {
+    if (u_in) io.add(u_in[q], fb, false);
+    if (u_out) io.add(u_out[q], fb, true);
+    if (far) io.add(far[q], db, true);
+    if (x0 && !(u_out && x0[q] == u_out[q])) io.add(x0[q], fb, false);   // x0[q] may be u_out[q]
+  }
+  const bool copy = !io.disjoint();
+  rc = load_rhs(P, f, n_views, u_in, x0, copy, (float2* const*)u_out, st);
   if (rc) return rc;
+  const bool far_direct = far && !copy && !P->pupil_h;
+  if (far_direct)
+    for (int q = 0; q < n_views; ++q) e.slots_h[q].far = (float2*)far[q];
   rc = engine_solve(P, n_views, st);
   if (rc) return rc;
   const int status = worst_status(e, n_views, stats);
@@ -1340,13 +1414,13 @@ static int forward_impl(ls_plan* P, const float* f, int n_views, const ls_c64* c
     seq_far(P, n_views, 0, st);
     rc = pupil_on_far(P, n_views, st);
     if (rc) return rc;
-    for (int q = 0; q < n_views; ++q)
-      LS_CUDA_TRY(cudaMemcpyAsync(far[q], e.far + (size_t)q * P->mx * P->my, (size_t)P->mx * P->my * sizeof(float2),
-                                  cudaMemcpyDeviceToDevice, st));
+    if (!far_direct)
+      for (int q = 0; q < n_views; ++q)
+        LS_CUDA_TRY(cudaMemcpyAsync(far[q], e.far + (size_t)q * P->mx * P->my, db, cudaMemcpyDeviceToDevice, st));
   }
   if (u_out)
-    for (int q = 0; q < n_views; ++q)
-      LS_CUDA_TRY(cudaMemcpyAsync(u_out[q], e.vptr(V_X, q), e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+    for (int q = 0; q < n_views && !rc; ++q) rc = store_field(e, q, u_out[q], st);
+  if (rc) return rc;
   LS_CUDA_TRY(cudaGetLastError());
   return status;
 }
@@ -1374,17 +1448,21 @@ int ls_farfield(ls_plan* P, const float* f, int n_views, const ls_c64* const* u,
   rc = engine_reserve(P, n_views);
   if (rc) return rc;
   Engine& e = P->eng;
+  // the fields are read, and (without a pupil) the far fields written, where they are: every field has
+  // been read before the first far field is written
   for (int q = 0; q < n_views; ++q) {
-    LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), u[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
-    slot_defaults(P, e.slots_h[q], f, 0);
+    slot_defaults(P, e.slots_h[q], q, f, 0);
+    e.slots_h[q].x = (const float2*)u[q];
+    if (!P->pupil_h) e.slots_h[q].far = (float2*)far[q];
   }
   LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, e.slots_h, (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
   seq_far(P, n_views, 0, st);
   rc = pupil_on_far(P, n_views, st);
   if (rc) return rc;
-  for (int q = 0; q < n_views; ++q)
-    LS_CUDA_TRY(cudaMemcpyAsync(far[q], e.far + (size_t)q * P->mx * P->my, (size_t)P->mx * P->my * sizeof(float2),
-                                cudaMemcpyDeviceToDevice, st));
+  if (P->pupil_h)
+    for (int q = 0; q < n_views; ++q)
+      LS_CUDA_TRY(cudaMemcpyAsync(far[q], e.far + (size_t)q * P->mx * P->my, (size_t)P->mx * P->my * sizeof(float2),
+                                  cudaMemcpyDeviceToDevice, st));
   LS_CUDA_TRY(cudaStreamSynchronize(st));
   return LS_OK;
 }
@@ -1404,11 +1482,13 @@ int ls_farfield_adjoint(ls_plan* P, int n_views, const ls_c64* const* r, ls_c64*
   if (rc) return rc;
   rc = engine_upload_ptrs(P, 1, rt.data(), n_views, st);
   if (rc) return rc;
-  for (int q = 0; q < n_views; ++q) slot_defaults(P, e.slots_h[q], nullptr, 1);
+  // the outputs are written last, where they are: every residual has been read by then
+  for (int q = 0; q < n_views; ++q) {
+    slot_defaults(P, e.slots_h[q], q, nullptr, 1);
+    e.slots_h[q].bo = (float2*)out[q];
+  }
   LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, e.slots_h, (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
   seq_far_adjoint(P, n_views, (const float2* const*)engine_ptr_table(P, 1), 0, st);
-  for (int q = 0; q < n_views; ++q)
-    LS_CUDA_TRY(cudaMemcpyAsync(out[q], e.vptr(V_B, q), e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
   LS_CUDA_TRY(cudaStreamSynchronize(st));
   return LS_OK;
 }
@@ -1511,16 +1591,15 @@ int ls_gradient(ls_plan* P, const float* f, int n_views, const ls_c64* const* u_
     // recompute the forward fields and keep them
     rc = engine_reserve_ucache(P, n_views);
     if (rc) return rc;
-    rc = load_rhs(P, f, n_views, u_in, 0, st);
+    std::vector<float2*> keep(n_views);
+    for (int q = 0; q < n_views; ++q) uptr[q] = keep[q] = e.ucache + (size_t)q * e.N;
+    rc = load_rhs(P, f, n_views, u_in, nullptr, false, keep.data(), st);
     if (rc) return rc;
     rc = engine_solve(P, n_views, st);
     if (rc) return rc;
     fwd_status = worst_status(e, n_views, nullptr);
-    for (int q = 0; q < n_views; ++q) {
-      LS_CUDA_TRY(cudaMemcpyAsync(e.ucache + (size_t)q * e.N, e.vptr(V_X, q), e.N * sizeof(float2),
-                                  cudaMemcpyDeviceToDevice, st));
-      uptr[q] = e.ucache + (size_t)q * e.N;
-    }
+    for (int q = 0; q < n_views && !rc; ++q) rc = store_field(e, q, keep[q], st);
+    if (rc) return rc;
   } else {
     for (int q = 0; q < n_views; ++q) uptr[q] = u_fwd[q];
   }
@@ -1530,11 +1609,12 @@ int ls_gradient(ls_plan* P, const float* f, int n_views, const ls_c64* const* u_
   if (rc) return rc;
   rc = engine_upload_ptrs(P, 1, rt.data(), n_views, st);
   if (rc) return rc;
-  for (int q = 0; q < n_views; ++q) slot_defaults(P, e.slots_h[q], f, 1);
+  for (int q = 0; q < n_views; ++q) {
+    slot_defaults(P, e.slots_h[q], q, f, 1);
+    e.slots_h[q].x = e.vptr(V_B, q);   // the initial guess is the right-hand side
+  }
   LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, e.slots_h, (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
   seq_far_adjoint(P, n_views, (const float2* const*)engine_ptr_table(P, 1), 0, st);
-  for (int q = 0; q < n_views; ++q)
-    LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), e.vptr(V_B, q), e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
   rc = engine_solve(P, n_views, st);
   if (rc) return rc;
   const int adj_status = worst_status(e, n_views, stats);
@@ -1544,7 +1624,7 @@ int ls_gradient(ls_plan* P, const float* f, int n_views, const ls_c64* const* u_
   std::vector<float> w(n_views);
   for (int q = 0; q < n_views; ++q) w[q] = view_weights ? (float)view_weights[q] : 1.0f;
   LS_CUDA_TRY(cudaMemcpyAsync(e.weights_d, w.data(), n_views * sizeof(float), cudaMemcpyHostToDevice, st));
-  GradParams g{e.N, n_views, (const float2* const*)engine_ptr_table(P, 2), e.vptr(V_X), e.N, e.weights_d, grad};
+  GradParams g{e.N, n_views, (const float2* const*)engine_ptr_table(P, 2), e.slots_d, e.weights_d, grad};
   launch_gradient(g, st);
   LS_CUDA_TRY(cudaGetLastError());
   LS_CUDA_TRY(cudaStreamSynchronize(st));

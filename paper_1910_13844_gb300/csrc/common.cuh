@@ -75,6 +75,12 @@ enum SlotFlag : unsigned {
 
 struct SlotDev {
   const float* f;      // potential of this slot's request (N floats)
+  // The slot's vectors that may live in the caller's memory (defaults: the workspace, slot_defaults)
+  const float2* b;     // right-hand side
+  const float2* x;     // current field: the initial guess (often b itself) until the first update, then xo
+  float2* xo;          // where updates write the field
+  float2* bo;          // G~^H r is written here (the adjoint right-hand side)
+  float2* far;         // G~ (f x) is written here
   unsigned flags;
   int adjoint;         // 1: operator x - G^H (f x)
   int first;           // 1: next p-update starts the recurrence (p = r)

@@ -33,10 +33,10 @@ struct Engine {
   int maxparts = 0;
   SlotDev* slots_d = nullptr;
   SlotDev* slots_h = nullptr;   // pinned mirror
-  int* counts_d = nullptr;      // [0..3] slot counts (k_count), [4] device error flag (a wait gave up)
+  int* counts_d = nullptr;      // [4] device error flag (a wait gave up), [6] work-unit counter (k_zwd)
   int* counts_h = nullptr;      // pinned
   void** ptrs_d = nullptr;      // pointer tables: [4][cap]
-  double* kvec_d = nullptr;     // [cap*6]: wave vectors, 3 per view (twice for the built-in plane waves)
+  double* kvec_d = nullptr;     // [cap*6]: wave vectors, 3 per view
   float* weights_d = nullptr;   // [cap]
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t iter_graph = nullptr;
@@ -120,8 +120,8 @@ int engine_reserve(ls_plan* P, int nslots);
 int engine_reserve_ucache(ls_plan* P, int nslots);
 void engine_release(Engine& e);
 
-// Upload host slot states [0, nslots) and run BiCGStab until every slot has
-// left SLOT_ITER/SLOT_RESID.  Vectors b and x must be set.
+// Upload host slot states [0, nslots) (SLOT_RESID set) and run BiCGStab until every slot has left
+// SLOT_ITER/SLOT_RESID.  Vectors b and x must be set.  Returns with the final states in slots_h.
 int engine_solve(ls_plan* P, int nslots, cudaStream_t st);
 // Sequences of kernel launches (no synchronisation).
 void seq_resid(ls_plan* P, int nslots, cudaStream_t st);
@@ -132,7 +132,8 @@ void seq_far(ls_plan* P, int nslots, unsigned mask, cudaStream_t st);
 void seq_far_adjoint(ls_plan* P, int nslots, const float2* const* r_dev_table, unsigned mask, cudaStream_t st);
 int engine_upload_ptrs(ls_plan* P, int table, const void* const* host_ptrs, int n, cudaStream_t st);
 void** engine_ptr_table(ls_plan* P, int table);
-void slot_defaults(const ls_plan* P, SlotDev& s, const float* f, int adjoint);
+// State of slot `slot` at the start of a solve, its vectors in the workspace.
+void slot_defaults(const ls_plan* P, SlotDev& s, int slot, const float* f, int adjoint);
 int ensure_iter_graph(ls_plan* P, int nslots);
 // Shallow view of slots [s0, s0 + n) of P's engine as slots [0, n) (no ownership).
 ls_plan plan_slot_view(const ls_plan* P, int s0);

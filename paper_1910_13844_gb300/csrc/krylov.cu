@@ -33,12 +33,13 @@ __global__ void __launch_bounds__(256, 4) k_update(UpdParams a) {
   const float4* s = reinterpret_cast<const float4*>(a.s + base);
   const float4* t = reinterpret_cast<const float4*>(a.t + base);
   const float4* rh = reinterpret_cast<const float4*>(a.rh + base);
-  float4* x = reinterpret_cast<float4*>(a.x + base);
+  const float4* xi = reinterpret_cast<const float4*>(sd.x);
+  float4* xo = reinterpret_cast<float4*>(sd.xo);
   float4* r = reinterpret_cast<float4*>(a.r + base);
   const size_t n4 = a.n / 2;
   float acc[3] = {0.f, 0.f, 0.f};
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    float4 pv = __ldg(p + i), sv = __ldg(s + i), tv = __ldg(t + i), hv = __ldg(rh + i), xv = x[i];
+    float4 pv = __ldg(p + i), sv = __ldg(s + i), tv = __ldg(t + i), hv = __ldg(rh + i), xv = xi[i];
     float2 p0 = make_float2(pv.x, pv.y), p1 = make_float2(pv.z, pv.w);
     float2 s0 = make_float2(sv.x, sv.y), s1 = make_float2(sv.z, sv.w);
     float2 t0 = make_float2(tv.x, tv.y), t1 = make_float2(tv.z, tv.w);
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(256, 4) k_update(UpdParams a) {
     float2 x1 = cadd(make_float2(xv.z, xv.w), cadd(cmul(al, p1), cmul(om, s1)));
     float2 r0 = csub(s0, cmul(om, t0));
     float2 r1 = csub(s1, cmul(om, t1));
-    x[i] = make_float4(x0.x, x0.y, x1.x, x1.y);
+    xo[i] = make_float4(x0.x, x0.y, x1.x, x1.y);
     r[i] = make_float4(r0.x, r0.y, r1.x, r1.y);
     float2 d0 = cdotterm(make_float2(hv.x, hv.y), r0);
     float2 d1 = cdotterm(make_float2(hv.z, hv.w), r1);
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(256) k_scalar(ScalarParams a) {
       const double2 rho_new = make_double2(s0, s1);   // <rh, r>
       const double rr = s2;
       sd.iters += 1;
+      sd.x = sd.xo;   // the update has written the field there
       sd.rnorm2 = rr;
       const double rel = sd.bnorm2 > 0.0 ? sqrt(rr / sd.bnorm2) : 0.0;
       if (!isfinite(rel)) {
@@ -188,20 +190,6 @@ __global__ void k_zero_shadow(const SlotDev* slots, int slot, float2* rh, size_t
   float2* v = rh + (size_t)slot * n;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     v[i] = make_float2(0.f, 0.f);
-}
-
-// Count slots per flag so the host can decide what to run next.
-__global__ void k_count(const SlotDev* slots, int nslots, int* out) {
-  __shared__ int c[4];
-  if (threadIdx.x < 4) c[threadIdx.x] = 0;
-  __syncthreads();
-  for (int s = threadIdx.x; s < nslots; s += blockDim.x) {
-    const unsigned f = slots[s].flags;
-    if (f & SLOT_ITER) atomicAdd(&c[0], 1);
-    if (f & SLOT_RESID) atomicAdd(&c[1], 1);
-  }
-  __syncthreads();
-  if (threadIdx.x < 4) out[threadIdx.x] = c[threadIdx.x];
 }
 
 // ------------------------------------------------------------------ element-wise kernels
@@ -296,7 +284,7 @@ __global__ void k_gradient(GradParams a) {
     float acc = 0.f;
     for (int s = 0; s < a.nslots; ++s) {
       const float2 u = __ldg(a.u[s] + i);
-      const float2 w = __ldg(a.w + (size_t)s * a.w_stride + i);
+      const float2 w = __ldg(a.slots[s].x + i);
       acc += a.c[s] * (u.x * w.x + u.y * w.y);
     }
     a.grad[i] = acc;
@@ -346,9 +334,6 @@ void launch_scalar(const ScalarParams& a, int nslots, cudaStream_t st) {
 }
 void launch_zero_shadow(const SlotDev* slots, int slot, float2* rh, size_t n, cudaStream_t st) {
   k_zero_shadow<<<256, 256, 0, st>>>(slots, slot, rh, n);
-}
-void launch_count(const SlotDev* slots, int nslots, int* out, cudaStream_t st) {
-  k_count<<<1, 256, 0, st>>>(slots, nslots, out);
 }
 cudaError_t launch_plane_waves(const PlaneWaveParams& a0, int nviews, cudaStream_t st) {
   PlaneWaveParams a = a0;

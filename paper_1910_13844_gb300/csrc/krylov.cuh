@@ -14,7 +14,7 @@ unsigned bounds_site_krylov(bool clear);
 struct UpdParams {
   SlotSel sel;
   size_t n, vstride;
-  float2 *x, *r;
+  float2* r;                // the field is read from the slot's x and written to its xo
   const float2 *p, *s, *t, *rh;
   double* partials;
   int maxparts = 0;   // partial-sum blocks allocated per slot (0: not checked)
@@ -56,7 +56,7 @@ struct GradParams {
   size_t n;
   int nslots;
   const float2* const* u;     // device array of forward fields
-  const float2* w; size_t w_stride;
+  const SlotDev* slots;       // the adjoint fields w_s = slots[s].x
   const float* c;             // device, per-slot weights
   float* grad;
 };
@@ -71,7 +71,6 @@ struct ResidualParams {
 
 void launch_update(const UpdParams& a, int nblocks, int nslots, cudaStream_t st);
 void launch_scalar(const ScalarParams& a, int nslots, cudaStream_t st);
-void launch_count(const SlotDev* slots, int nslots, int* out, cudaStream_t st);
 void launch_zero_shadow(const SlotDev* slots, int slot, float2* rh, size_t n, cudaStream_t st);
 void launch_inner(const ResidualParams& a, int nblocks, int nviews, cudaStream_t st);
 cudaError_t launch_plane_waves(const PlaneWaveParams& a, int nviews, cudaStream_t st);

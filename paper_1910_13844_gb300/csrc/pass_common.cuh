@@ -11,6 +11,7 @@
 namespace lsgpu {
 
 enum FxMode : int { FX_F_TIMES = 0, FX_COPY = 1, FX_BICG_P = 2, FX_BICG_S = 3 };
+enum IxOut : int { IX_OUT_XO = 0, IX_OUT_FAR = 1, IX_OUT_BO = 2 };
 enum IxMode : int { IX_STORE = 0, IX_MATVEC = 1, IX_BICG_V = 2, IX_BICG_T = 3, IX_RESID = 4 };
 
 struct SlotSel {
@@ -29,7 +30,7 @@ struct FxParams {
   SlotSel sel;
   int nx, rows;                // transform length is 2nx; rows = ny*nz pencils per slot
   int mode;
-  const float2* src;           // F_TIMES/COPY: vector; BICG_P/BICG_S: r
+  const float2* src;           // F_TIMES/COPY: vector (null: the slot's field x); BICG_P/BICG_S: r
   float2* vp;                  // BICG_P: p (read, then overwritten with the new p)
   const float2* vv;            // BICG_P/BICG_S: v
   float2* vs;                  // BICG_S: s (written)
@@ -85,9 +86,11 @@ struct IxParams {
   int nx, rows;                // input rows of length 2nx; output rows of length nx (or window)
   int mode;
   const float2* src; size_t src_stride;   // A1
-  const float2* in0;           // MATVEC: x; BICG_V: p; BICG_T: s; RESID: x
-  const float2* in1;           // BICG_V: rh; RESID: b
-  float2* out0;                // STORE/MATVEC: y; BICG_V: v; BICG_T: t; RESID: r
+  const float2* in0;           // MATVEC: x (null: the slot's x); BICG_V: p; BICG_T: s; RESID: null, the slot's x
+  const float2* in1;           // BICG_V: rh; RESID: null, the slot's b
+  float2* out0;                // STORE/MATVEC: y (null: the slot's xo, far or bo as out_slot says); BICG_V: v;
+                               // BICG_T: t; RESID: r
+  int out_slot = IX_OUT_XO;    // where a null out0 points
   float2* out1;                // RESID: rh (= r)
   size_t vstride;              // slot stride for in*/out* (STORE: stride of out0)
   int out_o, out_m;            // STORE: output window [out_o, out_o+out_m) of x; out rows are out_m long

@@ -105,6 +105,8 @@ __device__ __forceinline__ void fx_body(const FxParams& a) {
   const bool valid = row < a.rows;
   const size_t voff = (size_t)slot * a.vstride + (size_t)row * nx;
   const float* f = slot_f(a.sel, slot);
+  // element voff of the source (the slot's own vector where src is null)
+  const float2* src = a.src ? a.src + voff : a.sel.slots[slot].x + (size_t)row * nx;
   float2 v[R1];
 #pragma unroll
   for (int n1 = 0; n1 < R1; ++n1) v[n1] = make_float2(0.f, 0.f);
@@ -127,7 +129,7 @@ __device__ __forceinline__ void fx_body(const FxParams& a) {
       if (!LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)row * nx + x, (size_t)a.rows * nx, a.vstride),
                         BS_FX_VEC))
         continue;
-      float2 val = __ldg(a.src + i);
+      float2 val = __ldg(src + x);
       if (a.mode == FX_BICG_P) {
         if (!first) {
           // p = r + beta (p - omega v)
@@ -437,13 +439,17 @@ __device__ __forceinline__ void ix_body(const IxParams& a) {
   const int nx = L / 2;
   const int row = blockIdx.x * G::PC + p;
   const bool valid = row < a.rows;
+  // this slot's operands (its own vectors where the launch names none)
+  const size_t sbase = (size_t)slot * a.vstride;
+  const float2* in0 = a.in0 ? a.in0 + sbase : a.mode == IX_STORE ? nullptr : a.sel.slots[slot].x;
+  const float2* in1 = a.in1 ? a.in1 + sbase : a.mode == IX_RESID ? a.sel.slots[slot].b : nullptr;
   // the epilogue's operands are read after both transforms: ask L2 for their lines now (one
   // 128-byte line per thread and vector; a row holds nx/16 lines)
   if (a.prefetch && valid && a.mode != IX_STORE) {
     constexpr int lines = (L / 2) / 16;
-    const size_t voff0 = (size_t)slot * a.vstride + (size_t)row * nx;
-    if (t < lines) prefetch_l2(a.in0 + voff0 + 16 * t);
-    else if (t < 2 * lines && (a.mode == IX_BICG_V || a.mode == IX_RESID)) prefetch_l2(a.in1 + voff0 + 16 * (t - lines));
+    const size_t voff0 = (size_t)row * nx;
+    if (t < lines) prefetch_l2(in0 + voff0 + 16 * t);
+    else if (t < 2 * lines && (a.mode == IX_BICG_V || a.mode == IX_RESID)) prefetch_l2(in1 + voff0 + 16 * (t - lines));
   }
   // first stage: TR takes the CTA's rows along the lanes (see fx_store)
   const int tid = p * G::T + t;
@@ -478,12 +484,14 @@ __device__ __forceinline__ void ix_body(const IxParams& a) {
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) u[n2] = S[t * G::SROW + n2];
     Dft<R2, +1, R2, R2 / 2>::run(u);
-    const size_t voff = (size_t)slot * a.vstride + (size_t)row * nx;
+    float2* out0 = a.out0 ? a.out0 + sbase
+                   : a.out_slot == IX_OUT_XO ? a.sel.slots[slot].xo
+                   : a.out_slot == IX_OUT_FAR ? a.sel.slots[slot].far : a.sel.slots[slot].bo;
 #pragma unroll
     for (int k2 = 0; k2 < R2 / 2; ++k2) {
       const int x = t + R1 * k2;
       const float2 g = u[k2];
-      const size_t i = voff + x;
+      const size_t i = (size_t)row * nx + x;
       if (!LS_IN_BOUNDS(a.mode == IX_STORE ||
                             slot_elem_ok(slot, a.sel.nslots, (size_t)row * nx + x, (size_t)a.rows * nx, a.vstride),
                         BS_IX_VEC))
@@ -494,31 +502,31 @@ __device__ __forceinline__ void ix_body(const IxParams& a) {
           if (xo >= 0 && xo < a.out_m &&
               LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)row * a.out_m + xo, (size_t)a.rows * a.out_m,
                                         a.vstride), BS_IX_VEC))
-            a.out0[(size_t)slot * a.vstride + (size_t)row * a.out_m + xo] = g;
+            out0[(size_t)row * a.out_m + xo] = g;
         } break;
         case IX_MATVEC:
-          a.out0[i] = csub(__ldg(a.in0 + i), g);
+          out0[i] = csub(__ldg(in0 + i), g);
           break;
         case IX_BICG_V: {
-          float2 vv = csub(__ldg(a.in0 + i), g);
-          a.out0[i] = vv;
-          float2 d = cdotterm(__ldg(a.in1 + i), vv);   // conj(rh) v
+          float2 vv = csub(__ldg(in0 + i), g);
+          out0[i] = vv;
+          float2 d = cdotterm(__ldg(in1 + i), vv);   // conj(rh) v
           acc[0] += d.x; acc[1] += d.y;
           acc[2] += vv.x * vv.x + vv.y * vv.y;          // ||v||^2 (relative breakdown test)
         } break;
         case IX_BICG_T: {
-          float2 ss = __ldg(a.in0 + i);
+          float2 ss = __ldg(in0 + i);
           float2 tt = csub(ss, g);
-          a.out0[i] = tt;
+          out0[i] = tt;
           float2 d = cdotterm(tt, ss);                  // conj(t) s
           acc[0] += d.x; acc[1] += d.y;
           acc[2] += tt.x * tt.x + tt.y * tt.y;
         } break;
         case IX_RESID: {
-          float2 b = __ldg(a.in1 + i);
-          float2 r = cadd(csub(b, __ldg(a.in0 + i)), g);   // b - (x - G f x)
-          a.out0[i] = r;
-          a.out1[i] = r;
+          float2 b = __ldg(in1 + i);
+          float2 r = cadd(csub(b, __ldg(in0 + i)), g);   // b - (x - G f x)
+          out0[i] = r;
+          a.out1[sbase + i] = r;
           acc[0] += r.x * r.x + r.y * r.y;
           acc[1] += b.x * b.x + b.y * b.y;
         } break;

@@ -277,7 +277,7 @@ struct ls_server {
     }
     cudaMemcpyAsync(e.vptr(V_X, r->s0), e.vptr(V_B, r->s0), (size_t)r->n * e.N * sizeof(float2),
                     cudaMemcpyDeviceToDevice, st);
-    for (int q = 0; q < r->n; ++q) slot_defaults(P, e.slots_h[r->s0 + q], r->req.f, 0);
+    for (int q = 0; q < r->n; ++q) slot_defaults(P, e.slots_h[r->s0 + q], r->s0 + q, r->req.f, 0);
     upload_slots(l, r->s0, r->n);
     r->phase = PH_FWD;
     l->n_resid += r->n;
@@ -336,7 +336,7 @@ struct ls_server {
                     cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(e.vptr(V_X, r->s0), e.vptr(V_B, r->s0), (size_t)r->n * e.N * sizeof(float2),
                     cudaMemcpyDeviceToDevice, st);
-    for (int q = 0; q < r->n; ++q) slot_defaults(P, e.slots_h[r->s0 + q], r->req.f, 1);
+    for (int q = 0; q < r->n; ++q) slot_defaults(P, e.slots_h[r->s0 + q], r->s0 + q, r->req.f, 1);
     upload_slots(l, r->s0, r->n);
     r->phase = PH_ADJ;
     l->n_resid += r->n;
@@ -367,7 +367,7 @@ struct ls_server {
     r->ptrs.assign(r->n, nullptr);
     for (int q = 0; q < r->n; ++q) r->ptrs[q] = e.ucache + (size_t)(r->s0 + q) * e.N;
     cudaMemcpyAsync(engine_ptr_table(P, 2) + r->s0, r->ptrs.data(), r->n * sizeof(void*), cudaMemcpyHostToDevice, st);
-    GradParams g{e.N, r->n, (const float2* const*)(engine_ptr_table(P, 2) + r->s0), e.vptr(V_X, r->s0), e.N,
+    GradParams g{e.N, r->n, (const float2* const*)(engine_ptr_table(P, 2) + r->s0), e.slots_d + r->s0,
                  e.weights_d + r->s0, r->req.grad};
     launch_gradient(g, st);
     r->phase = PH_FINISHING;

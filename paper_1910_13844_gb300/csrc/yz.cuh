@@ -589,7 +589,7 @@ struct YzImpl {
     YzParams a = a0;
     a.sel.nslots = nslots;
     const int jobs = 2 * a.nx * nslots;
-    k_yz<NY, NZ><<<jobs < a.sms * W::MINB ? jobs : a.sms * W::MINB, W::NT, W::smem, st>>>(a);
+    k_yz<NY, NZ><<<imin(jobs, a.sms * W::MINB), W::NT, W::smem, st>>>(a);
   }
   static cudaError_t setup() {
     return cudaFuncSetAttribute(k_yz<NY, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W::smem);
