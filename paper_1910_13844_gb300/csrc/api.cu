@@ -508,7 +508,7 @@ void seq_resid(ls_plan* P, int nslots, cudaStream_t st) {
   matvec_core(P, sel, nslots, fx, ix, st);
   if (P->inj_zero_shadow_view >= 0 && P->inj_zero_shadow_view < nslots)
     launch_zero_shadow(e.slots_d, P->inj_zero_shadow_view, e.vptr(V_RH), e.N, st);
-  ScalarParams sc{e.slots_d, SLOT_RESID, PH_RESID, e.partials, ix_blocks(P)};
+  ScalarParams sc{e.slots_d, SLOT_RESID, PH_RESID, e.partials, ix_blocks(P), e.N};
   timed(P, LS_K_SCALAR, nslots, st, [&] { launch_scalar(sc, nslots, st); });
 }
 
@@ -531,7 +531,7 @@ void seq_iter(ls_plan* P, int nslots, cudaStream_t st) {
     ix.vstride = e.N;
     ix.partials = e.partials;
     matvec_core(P, sel, nslots, fx, ix, st);
-    ScalarParams sc{e.slots_d, SLOT_ITER, PH_ALPHA, e.partials, ix_blocks(P)};
+    ScalarParams sc{e.slots_d, SLOT_ITER, PH_ALPHA, e.partials, ix_blocks(P), e.N};
     timed(P, LS_K_SCALAR, nslots, st, [&] { launch_scalar(sc, nslots, st); });
   }
   // t = A s with s = r - alpha v
@@ -549,7 +549,7 @@ void seq_iter(ls_plan* P, int nslots, cudaStream_t st) {
     ix.vstride = e.N;
     ix.partials = e.partials;
     matvec_core(P, sel, nslots, fx, ix, st);
-    ScalarParams sc{e.slots_d, SLOT_ITER, PH_OMEGA, e.partials, ix_blocks(P)};
+    ScalarParams sc{e.slots_d, SLOT_ITER, PH_OMEGA, e.partials, ix_blocks(P), e.N};
     timed(P, LS_K_SCALAR, nslots, st, [&] { launch_scalar(sc, nslots, st); });
   }
   // x += alpha p + omega s ; r = s - omega t
@@ -564,7 +564,7 @@ void seq_iter(ls_plan* P, int nslots, cudaStream_t st) {
     u.maxparts = e.maxparts;
     const int nb = upd_blocks(P, nslots);
     timed(P, LS_K_UPDATE, nslots, st, [&] { launch_update(u, nb, nslots, st); });
-    ScalarParams sc{e.slots_d, SLOT_ITER, PH_RHO, e.partials, nb};
+    ScalarParams sc{e.slots_d, SLOT_ITER, PH_RHO, e.partials, nb, e.N};
     timed(P, LS_K_SCALAR, nslots, st, [&] { launch_scalar(sc, nslots, st); });
   }
 }

@@ -100,6 +100,42 @@ struct SlotDev {
   double rhnorm2;      // ||rh||^2 of the shadow residual (fixed from the last (re)start)
 };
 
+// ---------------------------------------------------------------- programmatic dependent launch
+//
+// The solver's kernels follow one another on one stream, many of them a few microseconds long.  On small
+// grids they let their CTAs be placed while the kernel before them drains (launch_pdl), and wait for that
+// kernel's completion before they touch memory (pdl_begin, the first statement of every CTA: a kernel
+// completes only after the one before it has).  Launched without the attribute the wait returns at once.
+// Small: below 2^20 voxels.  Measured without and with: forward at 32^3 x 1 292 -> 274 us, a served burst
+// at 64^3 12.5 -> 11.9 ms, gradient at 96^3 x 16 7.68 -> 7.62 ms; but 144^3 x 1 5.38 -> 5.41 ms, the operator
+// at 128^3 x 60 4.37 -> 4.52 ms.
+constexpr size_t kEarlyVoxels = (size_t)1 << 20;
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
+#ifdef __CUDACC__
+template <class... P, class... A>
+inline void launch_pdl(size_t voxels, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  if (voxels >= kEarlyVoxels) {
+    kernel<<<grid, block, smem, st>>>(args...);
+    return;
+  }
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, P(args)...);   // an error is left for the caller's cudaGetLastError
+}
+#endif
+
 // ---------------------------------------------------------------- error handling (host)
 
 void set_last_error(const char* fmt, ...);

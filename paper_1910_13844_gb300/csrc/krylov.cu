@@ -21,6 +21,7 @@ namespace lsgpu {
 // ------------------------------------------------------------------ update
 // x += alpha p + omega s ; r = s - omega t ; partials <rh, r>, ||r||^2
 __global__ void __launch_bounds__(256, 4) k_update(UpdParams a) {
+  pdl_begin();
   const int slot = blockIdx.y;
   if (!LS_IN_BOUNDS(slot < a.sel.nslots && (a.sel.nslots <= 1 || a.n <= a.vstride), BS_UPD_VEC)) return;
   if (!slot_runs(a.sel, slot)) return;
@@ -72,6 +73,7 @@ constexpr double kBreakdownRel = 1e-30;
 // One block per slot: sums the partials of the preceding kernel in a fixed
 // order (float64), then thread 0 advances the slot's BiCGStab state.
 __global__ void __launch_bounds__(256) k_scalar(ScalarParams a) {
+  pdl_begin();
   const int slot = blockIdx.x;
   SlotDev& sd = a.slots[slot];
   if (!(sd.flags & a.mask)) return;
@@ -239,6 +241,7 @@ __global__ void k_potential(const float* dn, size_t count, double eta_b, double 
 
 // Yhat[s][ky][kx] = sum_z K2hat[z][ky][kx] * A2[s][z][ky][kx]  (per-slice far-field kernels, eq. Gtild-1)
 __global__ void k_far_reduce(FarParams a) {
+  pdl_begin();
   const int slot = blockIdx.y;
   if (!slot_runs(a.sel, slot)) return;
   const size_t plane = (size_t)(2 * a.ny) * (2 * a.nx);
@@ -253,6 +256,7 @@ __global__ void k_far_reduce(FarParams a) {
 
 // A2[s][z][ky][kx] = conj(K2hat[z][ky][kx]) * Rhat[s][ky][kx]   (adjoint of the slice sum)
 __global__ void k_far_adjoint_mul(FarParams a) {
+  pdl_begin();
   const int slot = blockIdx.y;
   if (!slot_runs(a.sel, slot)) return;
   const size_t plane = (size_t)(2 * a.ny) * (2 * a.nx);
@@ -266,6 +270,7 @@ __global__ void k_far_adjoint_mul(FarParams a) {
 
 // plane[s][y][x] = r[s][y - oy][x - ox] inside the detector window, 0 outside
 __global__ void k_pad_detector(PadParams a) {
+  pdl_begin();
   const int slot = blockIdx.y;
   if (!slot_runs(a.sel, slot)) return;
   const size_t n = (size_t)a.ny * a.nx;
@@ -327,10 +332,10 @@ __global__ void __launch_bounds__(256) k_inner(ResidualParams a) {
 void launch_update(const UpdParams& a0, int nblocks, int nslots, cudaStream_t st) {
   UpdParams a = a0;
   a.sel.nslots = nslots;
-  k_update<<<dim3(nblocks, nslots), 256, 0, st>>>(a);
+  launch_pdl(a.n, k_update, dim3(nblocks, nslots), 256, 0, st, a);
 }
 void launch_scalar(const ScalarParams& a, int nslots, cudaStream_t st) {
-  k_scalar<<<nslots, 256, 0, st>>>(a);
+  launch_pdl(a.n, k_scalar, nslots, 256, 0, st, a);
 }
 void launch_zero_shadow(const SlotDev* slots, int slot, float2* rh, size_t n, cudaStream_t st) {
   k_zero_shadow<<<256, 256, 0, st>>>(slots, slot, rh, n);
@@ -357,19 +362,19 @@ void launch_potential(const float* dn, size_t count, double eta_b, double kb, fl
 }
 void launch_far_reduce(const FarParams& a, int nslots, cudaStream_t st) {
   const size_t plane = (size_t)(2 * a.ny) * (2 * a.nx);
-  k_far_reduce<<<dim3((unsigned)((plane + 255) / 256), nslots), 256, 0, st>>>(a);
+  launch_pdl((size_t)a.nx * a.ny * a.nz, k_far_reduce, dim3((unsigned)((plane + 255) / 256), nslots), 256, 0, st, a);
 }
 void launch_far_adjoint_mul(const FarParams& a, int nslots, cudaStream_t st) {
   const size_t total = (size_t)(2 * a.ny) * (2 * a.nx) * a.nz;
   int blocks = (int)((total + 255) / 256);
   if (blocks > 2432) blocks = 2432;
-  k_far_adjoint_mul<<<dim3(blocks, nslots), 256, 0, st>>>(a);
+  launch_pdl((size_t)a.nx * a.ny * a.nz, k_far_adjoint_mul, dim3(blocks, nslots), 256, 0, st, a);
 }
 void launch_pad_detector(const PadParams& a, int nslots, cudaStream_t st) {
   const size_t n = (size_t)a.ny * a.nx;
   int blocks = (int)((n + 255) / 256);
   if (blocks > 1024) blocks = 1024;
-  k_pad_detector<<<dim3(blocks, nslots), 256, 0, st>>>(a);
+  launch_pdl((size_t)a.nx * a.ny, k_pad_detector, dim3(blocks, nslots), 256, 0, st, a);
 }
 void launch_gradient(const GradParams& a, cudaStream_t st) {
   int blocks = (int)((a.n + 255) / 256);

@@ -26,6 +26,7 @@ struct ScalarParams {
   int phase;
   const double* partials;   // [slot][nparts][4]
   int nparts;
+  size_t n;                 // voxels per slot
 };
 
 struct PlaneWaveParams {

@@ -89,6 +89,7 @@ __device__ __forceinline__ void fx_store(const FxParams& a, const float2* sm, in
 // ------------------------------------------------------------------------- FX
 template <int L, bool TR>
 __device__ __forceinline__ void fx_body(const FxParams& a) {
+  pdl_begin();
   using G = Geo<L>;
   constexpr int R1 = G::R1, R2 = G::R2;
   extern __shared__ float2 sm[];
@@ -196,6 +197,7 @@ struct FXB {
 
 template <int L, bool TR>
 __device__ __forceinline__ void fxb_body(const FxParams& a) {
+  pdl_begin();
   using G = Geo<L>;
   using B = FXB<L>;
   constexpr int R1 = G::R1, R2 = G::R2, PC = G::PC, NX = B::NX, NSTG = B::NSTG;
@@ -345,6 +347,7 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 1) k_fxb_t(FxParams a)
 // with three; the other sizes keep the compiler's own register choice (k_strided).
 template <int L, int DIR, int P>
 __device__ __forceinline__ void strided_body(const StridedParams& a) {
+  pdl_begin();
   using G = Geo<L>;
   constexpr int R1 = G::R1, R2 = G::R2;
   extern __shared__ float2 sm[];
@@ -428,6 +431,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 
 template <int L, bool TR>
 __device__ __forceinline__ void ix_body(const IxParams& a) {
+  pdl_begin();
   using G = Geo<L>;
   constexpr int R1 = G::R1, R2 = G::R2;
   extern __shared__ float2 sm[];
@@ -577,8 +581,8 @@ struct PassImpl {
         FxParams b = a;
         b.sel.nslots = nslots;   // the kernel builds its list of active views from the selector
         const int grid = std::min(nrb * nslots, a.sms);
-        if (a.transposed) k_fxb_t<L><<<grid, dim3(G::T, G::PC), FXB<L>::smem, st>>>(b);
-        else k_fxb<L><<<grid, dim3(G::T, G::PC), FXB<L>::smem, st>>>(b);
+        if (a.transposed) launch_pdl((size_t)a.rows * (L / 2), k_fxb_t<L>, grid, dim3(G::T, G::PC), FXB<L>::smem, st, b);
+        else launch_pdl((size_t)a.rows * (L / 2), k_fxb<L>, grid, dim3(G::T, G::PC), FXB<L>::smem, st, b);
         return;
       }
     }
@@ -586,15 +590,15 @@ struct PassImpl {
     dim3 blk(G::T, G::PC), grd = a.views_fastest ? dim3(nslots, rbs) : dim3(rbs, nslots);
     FxParams b = a;
     b.sel.nslots = nslots;
-    if (a.transposed) k_fx_t<L><<<grd, blk, G::smem_contig, st>>>(b);
-    else k_fx<L><<<grd, blk, G::smem_contig, st>>>(b);
+    if (a.transposed) launch_pdl((size_t)a.rows * (L / 2), k_fx_t<L>, grd, blk, G::smem_contig, st, b);
+    else launch_pdl((size_t)a.rows * (L / 2), k_fx<L>, grd, blk, G::smem_contig, st, b);
   }
   static void ix(const IxParams& a0, int nslots, cudaStream_t st) {
     IxParams a = a0;
     a.sel.nslots = nslots;
     dim3 blk(G::T, G::PC), grd((a.rows + G::PC - 1) / G::PC, nslots);
-    if (a.transposed) k_ix_t<L><<<grd, blk, G::smem_contig, st>>>(a);
-    else k_ix<L><<<grd, blk, G::smem_contig, st>>>(a);
+    if (a.transposed) launch_pdl((size_t)a.rows * (L / 2), k_ix_t<L>, grd, blk, G::smem_contig, st, a);
+    else launch_pdl((size_t)a.rows * (L / 2), k_ix<L>, grd, blk, G::smem_contig, st, a);
   }
   template <int DIR>
   static void strided(const StridedParams& a0, int nslots, cudaStream_t st) {
@@ -604,15 +608,15 @@ struct PassImpl {
       constexpr int W = G::T * 32 <= 1024 ? 32 : 16;
       dim3 blk(W, G::T), grd(((a.ncont + W - 1) / W) * a.planes, nslots);
       if constexpr (StridedThree<L, W>::on)
-        k_strided3<L, DIR, W><<<grd, blk, (size_t)L * W * sizeof(float2), st>>>(a);
+        launch_pdl((size_t)a.planes * a.ncont / 2 * (L / 2), k_strided3<L, DIR, W>, grd, blk, (size_t)L * W * sizeof(float2), st, a);
       else
-        k_strided<L, DIR, W><<<grd, blk, (size_t)L * W * sizeof(float2), st>>>(a);
+        launch_pdl((size_t)a.planes * a.ncont / 2 * (L / 2), k_strided<L, DIR, W>, grd, blk, (size_t)L * W * sizeof(float2), st, a);
     } else {
       dim3 blk(G::PS, G::T), grd(((a.ncont + G::PS - 1) / G::PS) * a.planes, nslots);
       if constexpr (StridedThree<L, G::PS>::on)
-        k_strided3<L, DIR, G::PS><<<grd, blk, G::smem_strided, st>>>(a);
+        launch_pdl((size_t)a.planes * a.ncont / 2 * (L / 2), k_strided3<L, DIR, G::PS>, grd, blk, G::smem_strided, st, a);
       else
-        k_strided<L, DIR, G::PS><<<grd, blk, G::smem_strided, st>>>(a);
+        launch_pdl((size_t)a.planes * a.ncont / 2 * (L / 2), k_strided<L, DIR, G::PS>, grd, blk, G::smem_strided, st, a);
     }
   }
   static void fy(const StridedParams& a, int nslots, cudaStream_t st) { strided<-1>(a, nslots, st); }
@@ -631,7 +635,7 @@ struct PassImpl {
           a.nz <= 255) {
         const int ntiles = (2 * a.nx / ZWD<L>::P) * (2 * a.ny);
         cudaMemsetAsync(a.ctr, 0, sizeof(unsigned), st);
-        k_zwd<L><<<std::min(ntiles, a.sms * ZWD<L>::MINB), ZWD<L>::NT, ZWD<L>::smem, st>>>(a);
+        launch_pdl((size_t)a.nx * a.ny * a.nz, k_zwd<L>, std::min(ntiles, a.sms * ZWD<L>::MINB), ZWD<L>::NT, ZWD<L>::smem, st, a);
         return;
       }
     }
@@ -644,14 +648,14 @@ struct PassImpl {
       if (a.use_tma && (2 * a.nx) % ZG<L>::P == 0 && a.nz <= 256) {
         const int ntiles = (2 * a.nx / ZG<L>::P) * (2 * a.ny);
         if (a.persist && a.sms > 0)
-          k_zg<L, true><<<std::min(ntiles, a.sms * ZG<L>::MINB), ZG<L>::NT, ZG<L>::smem, st>>>(a);
+          launch_pdl((size_t)a.nx * a.ny * a.nz, k_zg<L, true>, std::min(ntiles, a.sms * ZG<L>::MINB), ZG<L>::NT, ZG<L>::smem, st, a);
         else
-          k_zg<L, false><<<ntiles, ZG<L>::NT, ZG<L>::smem, st>>>(a);
+          launch_pdl((size_t)a.nx * a.ny * a.nz, k_zg<L, false>, ntiles, ZG<L>::NT, ZG<L>::smem, st, a);
         return;
       }
     }
     dim3 blk(G::PS, G::T), grd(((2 * a.nx + G::PS - 1) / G::PS) * (2 * a.ny));
-    k_z<L><<<grd, blk, G::smem_z, st>>>(a);
+    launch_pdl((size_t)a.nx * a.ny * a.nz, k_z<L>, grd, blk, G::smem_z, st, a);
   }
   // persistent where the Green values live in registers: one wave of resident CTAs
   template <bool ALT>
@@ -660,11 +664,11 @@ struct PassImpl {
     const int ntiles = (2 * a.nx / W::P) * (2 * a.ny);
     if constexpr (W::GREG) {
       if (a.persist == 1 && a.sms > 0) {
-        k_zw<L, ALT, true><<<std::min(ntiles, a.sms * W::MINB), W::NT, W::smem, st>>>(a);
+        launch_pdl((size_t)a.nx * a.ny * a.nz, k_zw<L, ALT, true>, std::min(ntiles, a.sms * W::MINB), W::NT, W::smem, st, a);
         return;
       }
     }
-    k_zw<L, ALT, false><<<ntiles, W::NT, W::smem, st>>>(a);
+    launch_pdl((size_t)a.nx * a.ny * a.nz, k_zw<L, ALT, false>, ntiles, W::NT, W::smem, st, a);
   }
   template <bool ALT>
   static cudaError_t setup_zw() {

@@ -246,6 +246,7 @@ __device__ __forceinline__ void twiddle_out(const float2* v, unsigned taddr, con
 
 template <int NY, int NZ>
 __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParams a) {
+  pdl_begin();
   using W = YZ<NY, NZ>;
   constexpr int RA = W::RA, RB = W::RB, TY = W::TY, SA = W::SA, SB = W::SB, CSP = W::CSP, PZ = W::PZ;
   constexpr int R1 = W::R1, R2 = W::R2, TZ = W::TZ, S1 = W::S1, S2 = W::S2, XR = W::XR, CPW = W::CPW, NW = W::NW;
@@ -589,7 +590,7 @@ struct YzImpl {
     YzParams a = a0;
     a.sel.nslots = nslots;
     const int jobs = 2 * a.nx * nslots;
-    k_yz<NY, NZ><<<imin(jobs, a.sms * W::MINB), W::NT, W::smem, st>>>(a);
+    launch_pdl((size_t)a.nx * NY * NZ, k_yz<NY, NZ>, imin(jobs, a.sms * W::MINB), W::NT, W::smem, st, a);
   }
   static cudaError_t setup() {
     return cudaFuncSetAttribute(k_yz<NY, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W::smem);

@@ -26,6 +26,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // second staging buffer while the current view is transformed.
 template <int L>
 __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PS, Geo<L>::ZMINB) k_z(ZParams a) {
+  pdl_begin();
   using G = Geo<L>;
   constexpr int R1 = G::R1, R2 = G::R2, P = G::PS, NZ = L / 2;
   constexpr int NT = G::T * P;
@@ -442,6 +443,7 @@ __device__ __forceinline__ void zw_view(unsigned char* sb, float2* xc, const flo
 // form is faster depends on the views per launch (the autotuner times both).
 template <int L, bool ALT, bool PERSIST>
 __global__ void __launch_bounds__(ZW<L, ALT>::NT, ZW<L, ALT>::MINB) k_zw(const __grid_constant__ ZParams a) {
+  pdl_begin();
   using W = ZW<L, ALT>;
   static_assert(!PERSIST || W::GREG, "the persistent z pass keeps its Green values in registers");
   constexpr int R1 = W::R1, R2 = W::R2, P = W::P, NZ = W::NZ, CPW = W::CPW, T = W::T, NW = W::NW;
@@ -655,6 +657,7 @@ struct ZWD : ZWDL<L, ZWDL<L, 4>::fits ? 4 : 3> {};
 
 template <int L>
 __global__ void __launch_bounds__(ZWD<L>::NT, ZWD<L>::MINB) k_zwd(const __grid_constant__ ZParams a) {
+  pdl_begin();
   using W = ZWD<L>;
   constexpr int R1 = W::R1, R2 = W::R2, P = W::P, NZ = W::NZ, CPW = W::CPW, T = W::T, NW = W::NW, NS = W::NS;
   static_assert(W::ok, "k_zwd needs a register-resident Green split");
@@ -914,6 +917,7 @@ __device__ __forceinline__ bool group_all(int gi, bool v) {
 
 template <int L, bool PERSIST>
 __global__ void __launch_bounds__(ZG<L>::NT, ZG<L>::MINB) k_zg(const __grid_constant__ ZParams a) {
+  pdl_begin();
   using W = ZG<L>;
   constexpr int R1 = W::R1, R2 = W::R2, P = W::P, NZ = W::NZ, T = W::T, S1 = W::S1, CG = W::CG, WG = W::WG,
                 NW = W::NW, NS = W::NS, RA = W::RA, RB = W::RB;
