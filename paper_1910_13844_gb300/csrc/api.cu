@@ -581,6 +581,22 @@ void seq_iter_chunked(ls_plan* P, int nslots, cudaStream_t st) {
   }
 }
 
+// Far-field passes over nslots views: slices summed in chunks of at least eight, as many as fill the SMs.  The
+// partial planes (4 nx ny entries) go to A1, which holds nz / 2 of them.
+static FarPassParams far_base(ls_plan* P, SlotSel sel, int nslots) {
+  FarPassParams a;
+  memset(&a, 0, sizeof(a));
+  a.sel = sel;
+  a.ncont = 2 * P->nx;
+  a.ny = P->ny;
+  a.nz = P->nz;
+  const long long ctas = (long long)nslots * ((4LL * P->nx * P->ny + 255) / 256);   // of the sum, eight per SM
+  a.zchunks = (int)std::max(1LL, std::min((long long)P->nz / 8, (8LL * P->sms + ctas - 1) / ctas));
+  a.k2 = P->k2hat;
+  a.tw = P->tw_y;
+  return a;
+}
+
 // G~ (f x_s) for the selected slots, into their far buffers (eq. Gtild-1)
 void seq_far(ls_plan* P, int nslots, unsigned mask, cudaStream_t st) {
   Engine& e = P->eng;
@@ -590,19 +606,15 @@ void seq_far(ls_plan* P, int nslots, unsigned mask, cudaStream_t st) {
   timed(P, LS_K_FX, nslots, st, [&] { P->px.fx(fx, nslots, st); });
   StridedParams fy = fy_base(P, sel, e.a1, e.a1_stride, e.a2, e.a2_stride, P->nz);
   timed(P, LS_K_FY, nslots, st, [&] { P->py.fy(fy, nslots, st); });
-  FarParams fr;
-  memset(&fr, 0, sizeof(fr));
-  fr.sel = sel;
-  fr.nx = P->nx; fr.ny = P->ny; fr.nz = P->nz;
-  fr.a2 = e.a2; fr.a2_stride = e.a2_stride;
-  fr.k2 = P->k2hat;
-  fr.out = e.a1; fr.out_stride = e.a1_stride;
+  FarPassParams fr = far_base(P, sel, nslots);
+  fr.src = e.a2; fr.src_stride = e.a2_stride;
+  fr.dst = e.a1; fr.dst_stride = e.a1_stride;
   timed(P, LS_K_FAR, nslots, st, [&] { launch_far_reduce(fr, nslots, st); });
-  // 2-D inverse transform of the single plane, cropped to the detector window
-  StridedParams iy = fy_base(P, sel, e.a1, e.a1_stride, e.a2, e.a2_stride, 1);
-  iy.src_plane = 0; iy.dst_plane = 0;
-  iy.out_o = P->oy; iy.out_m = P->my;
-  timed(P, LS_K_FAR, nslots, st, [&] { P->py.iy(iy, nslots, st); });
+  // 2-D inverse transform of the summed plane, cropped to the detector window
+  fr.src = e.a1; fr.src_stride = e.a1_stride;
+  fr.dst = e.a2; fr.dst_stride = e.a2_stride;
+  fr.out_o = P->oy; fr.out_m = P->my;
+  timed(P, LS_K_FAR, nslots, st, [&] { P->py.far_sum(fr, nslots, st); });
   IxParams ix;
   memset(&ix, 0, sizeof(ix));
   ix.sel = sel;
@@ -636,25 +648,18 @@ void seq_far_adjoint(ls_plan* P, int nslots, const float2* const* r_dev_table, u
   timed(P, LS_K_FAR, nslots, st, [&] { P->px.fx(fx, nslots, st); });
   StridedParams fy = fy_base(P, sel, e.a2, e.a2_stride, e.a1, e.a1_stride, 1);
   timed(P, LS_K_FAR, nslots, st, [&] { P->py.fy(fy, nslots, st); });
-  FarParams fr;
-  memset(&fr, 0, sizeof(fr));
-  fr.sel = sel;
-  fr.nx = P->nx; fr.ny = P->ny; fr.nz = P->nz;
-  fr.a2 = e.a2; fr.a2_stride = e.a2_stride;
-  fr.k2 = P->k2hat;
-  fr.rhat = e.a1; fr.rhat_stride = e.a1_stride;
-  timed(P, LS_K_FAR, nslots, st, [&] { launch_far_adjoint_mul(fr, nslots, st); });
-  StridedParams iy = fy_base(P, sel, e.a2, e.a2_stride, e.a1, e.a1_stride, P->nz);
-  iy.src_plane = (size_t)2 * P->ny * 2 * P->nx;
-  iy.dst_plane = (size_t)P->ny * 2 * P->nx;
-  timed(P, LS_K_IY, nslots, st, [&] { P->py.iy(iy, nslots, st); });
+  // conj(K2hat_z) times that plane, inverse y transforms: the slices, in A2 as [nz][ny][2nx]
+  FarPassParams fr = far_base(P, sel, nslots);
+  fr.src = e.a1; fr.src_stride = e.a1_stride;
+  fr.dst = e.a2; fr.dst_stride = e.a2_stride;
+  timed(P, LS_K_IY, nslots, st, [&] { P->py.far_iy(fr, nslots, st); });
   IxParams ix;
   memset(&ix, 0, sizeof(ix));
   ix.sel = sel;
   ix.mode = IX_STORE;
   ix.nx = P->nx;
   ix.rows = P->ny * P->nz;
-  ix.src = e.a1; ix.src_stride = e.a1_stride;
+  ix.src = e.a2; ix.src_stride = e.a2_stride;
   ix.out_slot = IX_OUT_BO;
   ix.vstride = e.N;
   ix.out_o = 0; ix.out_m = P->nx;
@@ -878,37 +883,32 @@ void prof_resolve(ls_plan* P, bool wait) {
   pr.pending.resize(keep);
 }
 
-// far[q] <- P far[q] for the engine's detector buffers of slots [0, n) (no-op without a pupil)
-static int pupil_on_far(ls_plan* P, int n, cudaStream_t st) {
+// far[q] <- P e.far[q] for slots [0, n) (no-op without a pupil).  The A1 buffers (16 nz bytes for each of the
+// 2 nx ny columns of a slot's plane) are free once the far field is done and hold the scratch planes.
+static int pupil_on_far(ls_plan* P, int n, ls_c64* const* far, cudaStream_t st) {
   if (!P->pupil_h) return LS_OK;
-  double2* scratch = nullptr;
-  LS_CUDA_TRY(cudaMallocAsync((void**)&scratch, (size_t)4 * P->mx * P->my * sizeof(double2), st));
-  const size_t M = (size_t)P->mx * P->my;
-  int rc = LS_OK;
-  for (int q = 0; q < n && rc == LS_OK; ++q)
-    rc = apply_pupil_device(P, P->eng.far + q * M, P->eng.far + q * M, 0, scratch, st);
-  LS_CUDA_TRY(cudaFreeAsync(scratch, st));
-  return rc;
+  Engine& e = P->eng;
+  std::vector<const void*> src(n);
+  for (int q = 0; q < n; ++q) src[q] = e.far + (size_t)q * P->mx * P->my;
+  int rc = engine_upload_ptrs(P, 2, src.data(), n, st);
+  if (rc == LS_OK) rc = engine_upload_ptrs(P, 3, (const void* const*)far, n, st);
+  if (rc) return rc;
+  return apply_pupil_views(P, n, (const float2* const*)engine_ptr_table(P, 2), (float2* const*)engine_ptr_table(P, 3),
+                           0, e.a1, st);
 }
 
-// r'_q = P^H r_q into the engine's detector buffers (returns a host table of their pointers in tab)
-static int pupil_adjoint_residuals(ls_plan* P, int n, const ls_c64* const* r, std::vector<const void*>& tab,
-                                   cudaStream_t st) {
-  tab.assign(n, nullptr);
-  const size_t M = (size_t)P->mx * P->my;
-  if (!P->pupil_h) {
-    for (int q = 0; q < n; ++q) tab[q] = r[q];
-    return LS_OK;
-  }
-  double2* scratch = nullptr;
-  LS_CUDA_TRY(cudaMallocAsync((void**)&scratch, (size_t)4 * M * sizeof(double2), st));
-  int rc = LS_OK;
-  for (int q = 0; q < n && rc == LS_OK; ++q) {
-    rc = apply_pupil_device(P, (const float2*)r[q], P->eng.far + q * M, 1, scratch, st);
-    tab[q] = P->eng.far + q * M;
-  }
-  LS_CUDA_TRY(cudaFreeAsync(scratch, st));
-  return rc;
+// Uploads the table (1) of the residuals that G~^H is applied to: r_q, or P^H r_q in the engine's detector
+// buffers.
+static int pupil_adjoint_residuals(ls_plan* P, int n, const ls_c64* const* r, cudaStream_t st) {
+  if (!P->pupil_h) return engine_upload_ptrs(P, 1, (const void* const*)r, n, st);
+  Engine& e = P->eng;
+  std::vector<const void*> dst(n);
+  for (int q = 0; q < n; ++q) dst[q] = e.far + (size_t)q * P->mx * P->my;
+  int rc = engine_upload_ptrs(P, 3, (const void* const*)r, n, st);
+  if (rc == LS_OK) rc = engine_upload_ptrs(P, 1, dst.data(), n, st);
+  if (rc) return rc;
+  return apply_pupil_views(P, n, (const float2* const*)engine_ptr_table(P, 3), (float2* const*)engine_ptr_table(P, 1),
+                           1, e.a1, st);
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -1412,9 +1412,9 @@ static int forward_impl(ls_plan* P, const float* f, int n_views, const ls_c64* c
   const int status = worst_status(e, n_views, stats);
   if (far) {
     seq_far(P, n_views, 0, st);
-    rc = pupil_on_far(P, n_views, st);
+    rc = pupil_on_far(P, n_views, far, st);
     if (rc) return rc;
-    if (!far_direct)
+    if (!far_direct && !P->pupil_h)
       for (int q = 0; q < n_views; ++q)
         LS_CUDA_TRY(cudaMemcpyAsync(far[q], e.far + (size_t)q * P->mx * P->my, db, cudaMemcpyDeviceToDevice, st));
   }
@@ -1457,12 +1457,8 @@ int ls_farfield(ls_plan* P, const float* f, int n_views, const ls_c64* const* u,
   }
   LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, e.slots_h, (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
   seq_far(P, n_views, 0, st);
-  rc = pupil_on_far(P, n_views, st);
+  rc = pupil_on_far(P, n_views, far, st);
   if (rc) return rc;
-  if (P->pupil_h)
-    for (int q = 0; q < n_views; ++q)
-      LS_CUDA_TRY(cudaMemcpyAsync(far[q], e.far + (size_t)q * P->mx * P->my, (size_t)P->mx * P->my * sizeof(float2),
-                                  cudaMemcpyDeviceToDevice, st));
   LS_CUDA_TRY(cudaStreamSynchronize(st));
   return LS_OK;
 }
@@ -1477,10 +1473,7 @@ int ls_farfield_adjoint(ls_plan* P, int n_views, const ls_c64* const* r, ls_c64*
   rc = engine_reserve(P, n_views);
   if (rc) return rc;
   Engine& e = P->eng;
-  std::vector<const void*> rt;
-  rc = pupil_adjoint_residuals(P, n_views, r, rt, st);
-  if (rc) return rc;
-  rc = engine_upload_ptrs(P, 1, rt.data(), n_views, st);
+  rc = pupil_adjoint_residuals(P, n_views, r, st);
   if (rc) return rc;
   // the outputs are written last, where they are: every residual has been read by then
   for (int q = 0; q < n_views; ++q) {
@@ -1604,10 +1597,7 @@ int ls_gradient(ls_plan* P, const float* f, int n_views, const ls_c64* const* u_
     for (int q = 0; q < n_views; ++q) uptr[q] = u_fwd[q];
   }
   // adjoint right-hand sides b_q = G~^H P^H r_q
-  std::vector<const void*> rt;
-  rc = pupil_adjoint_residuals(P, n_views, residuals, rt, st);
-  if (rc) return rc;
-  rc = engine_upload_ptrs(P, 1, rt.data(), n_views, st);
+  rc = pupil_adjoint_residuals(P, n_views, residuals, st);
   if (rc) return rc;
   for (int q = 0; q < n_views; ++q) {
     slot_defaults(P, e.slots_h[q], q, f, 1);

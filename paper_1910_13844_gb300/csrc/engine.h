@@ -144,8 +144,11 @@ ls_plan* plan_clone_shared(const ls_plan* P);
 int tune_matvec(ls_plan* P, const float* f, int n, cudaStream_t st);
 // a forward solve of slots [0, n) from the right-hand sides already in V_B (x0 = b), for the autotuner
 int tune_forward(ls_plan* P, const float* f, int n, cudaStream_t st);
-// P y (adjoint: P^H y) for one detector field; scratch holds 4 my mx double2
-int apply_pupil_device(ls_plan* P, const float2* in, float2* out, int adjoint, double2* scratch, cudaStream_t st);
+// out[q] = P in[q] (adjoint: P^H in[q]) for n detector fields (device tables of their pointers; in may be out);
+// scratch holds pupil_scratch_bytes(P, n)
+int apply_pupil_views(ls_plan* P, int n, const float2* const* in, float2* const* out, int adjoint, void* scratch,
+                      cudaStream_t st);
+size_t pupil_scratch_bytes(const ls_plan* P, int n);
 
 // ls_matvec_noalloc set-up (noalloc.cu): the device address of the static scratch array on the
 // current device; loads the array's module (reserving the array) if that has not happened yet.

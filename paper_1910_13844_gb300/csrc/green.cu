@@ -6,6 +6,8 @@
 // Both are stored as complex64 for the hot path.
 #include "green.cuh"
 
+#include "fft64.cuh"
+
 #include <math.h>
 
 #include <map>
@@ -192,70 +194,16 @@ __global__ void k_to_c64(const double2* src, float2* dst, size_t n, double scale
 }
 
 // -------------------------------------------------------------- float64 FFT (plan time)
-// One CTA per pencil; the pencil (length L = 2^a 3^b, L <= 1024) is staged in
-// shared memory and transformed in place by Stockham autosort stages of radix
-// 4, 2 and 3.  dir = -1 forward, +1 inverse (unnormalised).
-__device__ __forceinline__ void zdft(double2* v, int r, int dir) {
-  if (r == 2) {
-    double2 t = v[1];
-    v[1] = zsub(v[0], t);
-    v[0] = zadd(v[0], t);
-  } else if (r == 4) {
-    double2 s0 = zadd(v[0], v[2]), d0 = zsub(v[0], v[2]);
-    double2 s1 = zadd(v[1], v[3]), d1 = zsub(v[1], v[3]);
-    double2 d1r = dir < 0 ? make_double2(d1.y, -d1.x) : make_double2(-d1.y, d1.x);
-    v[0] = zadd(s0, s1);
-    v[2] = zsub(s0, s1);
-    v[1] = zadd(d0, d1r);
-    v[3] = zsub(d0, d1r);
-  } else {  // 3
-    const double h = 0.86602540378443864676;
-    double2 s = zadd(v[1], v[2]), d = zsub(v[1], v[2]);
-    double2 m = make_double2(v[0].x - 0.5 * s.x, v[0].y - 0.5 * s.y);
-    double2 rr = dir < 0 ? make_double2(h * d.y, -h * d.x) : make_double2(-h * d.y, h * d.x);
-    v[0] = zadd(v[0], s);
-    v[1] = zadd(m, rr);
-    v[2] = zsub(m, rr);
-  }
-}
-
+// One CTA per pencil, staged in shared memory (fft64.cuh).  dir = -1 forward, +1 inverse (unnormalised).
 __global__ void k_fft64(double2* data, int L, size_t elem_stride, int ninner, size_t inner_stride,
                         size_t outer_stride, int dir, const double2* __restrict__ tw) {
   extern __shared__ double2 zb[];
-  double2* b0 = zb;
-  double2* b1 = zb + L;
   const size_t pencil = blockIdx.x;
   const size_t base = (pencil / ninner) * outer_stride + (pencil % ninner) * inner_stride;
-  for (int i = threadIdx.x; i < L; i += blockDim.x) b0[i] = data[base + (size_t)i * elem_stride];
+  for (int i = threadIdx.x; i < L; i += blockDim.x) zb[i] = data[base + (size_t)i * elem_stride];
   __syncthreads();
-  int rest = L, Ns = 1;
-  double2* src = b0;
-  double2* dst = b1;
-  while (rest > 1) {
-    const int r = (rest % 4 == 0) ? 4 : (rest % 2 == 0 ? 2 : 3);
-    const int m = L / r;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-      const int k = j % Ns;
-      double2 v[4];
-      for (int q = 0; q < r; ++q) {
-        v[q] = src[j + q * m];
-        if (q > 0) {
-          // exp(dir 2 pi i k q / (Ns r)) = tw[k q L / (Ns r)] (conjugated for dir = +1)
-          double2 w = tw[(size_t)k * q * (L / (Ns * r)) % L];
-          if (dir > 0) w.y = -w.y;
-          v[q] = zmul(v[q], w);
-        }
-      }
-      zdft(v, r, dir);
-      const int o = (j / Ns) * Ns * r + k;
-      for (int q = 0; q < r; ++q) dst[o + q * Ns] = v[q];
-    }
-    __syncthreads();
-    double2* tmp = src; src = dst; dst = tmp;
-    Ns *= r;
-    rest /= r;
-  }
-  for (int i = threadIdx.x; i < L; i += blockDim.x) data[base + (size_t)i * elem_stride] = src[i];
+  const double2* out = fft64_staged(zb, zb + L, L, 1, dir, tw, threadIdx.x, blockDim.x);
+  for (int i = threadIdx.x; i < L; i += blockDim.x) data[base + (size_t)i * elem_stride] = out[i];
 }
 
 // exp(-2 pi i j / L), j < L, in float64
@@ -269,7 +217,7 @@ __global__ void k_twiddle64(int L, double2* w) {
 
 // Twiddle table of length L on the current device, built on first use and kept for the process
 // (a few KB per length); the first build is synchronous so every stream may read it.
-static const double2* twiddle64(int L, cudaStream_t st) {
+const double2* twiddle64(int L, cudaStream_t st) {
   static std::mutex mu;
   static std::map<std::pair<int, int>, double2*> cache;
   int dev = 0;

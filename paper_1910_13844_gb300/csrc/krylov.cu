@@ -239,33 +239,24 @@ __global__ void k_potential(const float* dn, size_t count, double eta_b, double 
   }
 }
 
-// Yhat[s][ky][kx] = sum_z K2hat[z][ky][kx] * A2[s][z][ky][kx]  (per-slice far-field kernels, eq. Gtild-1)
-__global__ void k_far_reduce(FarParams a) {
+// Partial sums over a chunk of slices of K2hat[z][ky][kx] A2[s][z][ky][kx] (per-slice far-field kernels, eq. Gtild-1);
+// grid (views, blocks of the plane, chunks): views fastest, so that K2hat is read from L2 (192^3 x 8, where it is
+// larger than L2: 51 -> 42 us a view), chunks so that few views still fill the SMs (128^3 x 1: 67 -> 48 us).
+__global__ void __launch_bounds__(256) k_far_reduce(FarPassParams a) {
   pdl_begin();
-  const int slot = blockIdx.y;
+  const int slot = blockIdx.x;
   if (!slot_runs(a.sel, slot)) return;
-  const size_t plane = (size_t)(2 * a.ny) * (2 * a.nx);
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  const size_t plane = (size_t)(2 * a.ny) * a.ncont;
+  const size_t i = blockIdx.y * (size_t)blockDim.x + threadIdx.x;
   if (i >= plane) return;
-  const float2* src = a.a2 + (size_t)slot * a.a2_stride + i;
+  const int per = (a.nz + a.zchunks - 1) / a.zchunks;
+  const int z0 = blockIdx.z * per, z1 = min(a.nz, z0 + per);
+  const float2* src = a.src + (size_t)slot * a.src_stride + i;
   const float2* k = a.k2 + i;
   float2 acc = make_float2(0.f, 0.f);
-  for (int z = 0; z < a.nz; ++z) acc = cadd(acc, cmul(__ldg(k + (size_t)z * plane), __ldg(src + (size_t)z * plane)));
-  a.out[(size_t)slot * a.out_stride + i] = acc;
-}
-
-// A2[s][z][ky][kx] = conj(K2hat[z][ky][kx]) * Rhat[s][ky][kx]   (adjoint of the slice sum)
-__global__ void k_far_adjoint_mul(FarParams a) {
-  pdl_begin();
-  const int slot = blockIdx.y;
-  if (!slot_runs(a.sel, slot)) return;
-  const size_t plane = (size_t)(2 * a.ny) * (2 * a.nx);
-  const size_t total = plane * a.nz;
-  const float2* rhat = a.rhat + (size_t)slot * a.rhat_stride;
-  float2* dst = a.a2 + (size_t)slot * a.a2_stride;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    dst[i] = cmulc(__ldg(rhat + (i % plane)), __ldg(a.k2 + i));
-  }
+#pragma unroll 8
+  for (int z = z0; z < z1; ++z) acc = cadd(acc, cmul(__ldg(k + (size_t)z * plane), __ldg(src + (size_t)z * plane)));
+  a.dst[(size_t)slot * a.dst_stride + blockIdx.z * plane + i] = acc;
 }
 
 // plane[s][y][x] = r[s][y - oy][x - ox] inside the detector window, 0 outside
@@ -360,15 +351,10 @@ void launch_potential(const float* dn, size_t count, double eta_b, double kb, fl
   if (blocks < 1) blocks = 1;
   k_potential<<<blocks, 256, 0, st>>>(dn, count, eta_b, kb, f);
 }
-void launch_far_reduce(const FarParams& a, int nslots, cudaStream_t st) {
-  const size_t plane = (size_t)(2 * a.ny) * (2 * a.nx);
-  launch_pdl((size_t)a.nx * a.ny * a.nz, k_far_reduce, dim3((unsigned)((plane + 255) / 256), nslots), 256, 0, st, a);
-}
-void launch_far_adjoint_mul(const FarParams& a, int nslots, cudaStream_t st) {
-  const size_t total = (size_t)(2 * a.ny) * (2 * a.nx) * a.nz;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 2432) blocks = 2432;
-  launch_pdl((size_t)a.nx * a.ny * a.nz, k_far_adjoint_mul, dim3(blocks, nslots), 256, 0, st, a);
+void launch_far_reduce(const FarPassParams& a, int nslots, cudaStream_t st) {
+  const size_t plane = (size_t)(2 * a.ny) * a.ncont;
+  launch_pdl((size_t)a.ny * a.nz * a.ncont / 2, k_far_reduce, dim3(nslots, (unsigned)((plane + 255) / 256), a.zchunks), 256,
+             0, st, a);
 }
 void launch_pad_detector(const PadParams& a, int nslots, cudaStream_t st) {
   const size_t n = (size_t)a.ny * a.nx;

@@ -37,15 +37,6 @@ struct PlaneWaveParams {
   float2* tables = nullptr; // per-view 1-D phase factors (allocated by the launcher)
 };
 
-struct FarParams {
-  SlotSel sel;
-  int nx, ny, nz;
-  float2* a2; size_t a2_stride;           // reduce: input slices; adjoint: output
-  const float2* k2;                       // [nz][2ny][2nx], scaled by 1/(4 nx ny)
-  float2* out; size_t out_stride;         // reduce output [2ny][2nx] per slot
-  const float2* rhat; size_t rhat_stride; // adjoint input [2ny][2nx] per slot
-};
-
 struct PadParams {
   SlotSel sel;
   int nx, ny, mx, my, ox, oy;
@@ -76,8 +67,7 @@ void launch_zero_shadow(const SlotDev* slots, int slot, float2* rh, size_t n, cu
 void launch_inner(const ResidualParams& a, int nblocks, int nviews, cudaStream_t st);
 cudaError_t launch_plane_waves(const PlaneWaveParams& a, int nviews, cudaStream_t st);
 void launch_potential(const float* dn, size_t count, double eta_b, double kb, float* f, cudaStream_t st);
-void launch_far_reduce(const FarParams& a, int nslots, cudaStream_t st);
-void launch_far_adjoint_mul(const FarParams& a, int nslots, cudaStream_t st);
+void launch_far_reduce(const FarPassParams& a, int nslots, cudaStream_t st);
 void launch_pad_detector(const PadParams& a, int nslots, cudaStream_t st);
 void launch_gradient(const GradParams& a, cudaStream_t st);
 void launch_residual(const ResidualParams& a, int nblocks, int nviews, cudaStream_t st);

@@ -58,6 +58,18 @@ struct StridedParams {
   int wide = 0;                // 32 pencils per CTA instead of 16 (autotuned)
 };
 
+// The far field's passes over the slice spectra (planes of 2nx * 2ny entries)
+struct FarPassParams {
+  SlotSel sel;
+  int ncont, ny, nz;           // 2nx, rows of a slice, slices
+  int zchunks;                 // slices are summed in this many chunks, one partial plane each
+  const float2* src; size_t src_stride;   // far_reduce: A2 [slot][nz][2ny][2nx]; far_sum: partial planes; far_iy: Rhat
+  float2* dst; size_t dst_stride;         // far_reduce: partial planes [slot][zchunks][2ny][2nx]; else [..][ny][2nx]
+  const float2* k2;            // K2hat [nz][2ny][2nx]
+  const float2* tw;            // tw[j] = exp(-2 pi i j / L)
+  int out_o, out_m;            // far_sum: cropped output window of y
+};
+
 struct ZParams {
   CUtensorMap tmap;            // A2 of all slots as floats [slot][nz][2ny][4nx], box {32, 1, nz, 1}, 128B swizzle
   CUtensorMap gmap;            // x-unfolded Green array as floats [nz+1][ny+1][4nx], box {32, 1, nz+1}, 128B swizzle

@@ -424,6 +424,66 @@ template <int L, int DIR, int P>
 __global__ void __launch_bounds__(Geo<L>::T * P, 3) k_strided3(const StridedParams a) { strided_body<L, DIR, P>(a); }
 template <int L, int P> struct StridedThree { static constexpr bool on = Geo<L>::T * P > 256 && Geo<L>::T * P <= 384; };
 
+// ------------------------------------------------------------------------- far field
+// The far field sums K2hat_z times the 2-D spectrum of every slice (k_far_reduce, krylov.cu), its adjoint spreads
+// one spectrum over the slices times conj(K2hat_z): the product is part of the inverse y pass, so the products
+// (32N bytes written and 32N read per view) are never stored: 38 -> 15 us a view at 128^3 x 60.  (The sum as part
+// of the forward y pass, accumulated in registers slice by slice, was latency-bound: 27 us against 27 for FY and
+// the sum as two launches, each at the copy bandwidth.)  K2hat, shared by all views, comes from L2 where their CTAs
+// run together: views fastest in the grid.
+
+// Inverse y transform of one plane per CTA column tile.  ADJ: of conj(K2hat_z) Rhat, z = blockIdx.z, all ny rows
+// stored; else of the sum of the partial planes, the rows of the window [out_o, out_o + out_m).
+template <int L, bool ADJ>
+__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PS) k_far_iy(FarPassParams a) {
+  pdl_begin();
+  using G = Geo<L>;
+  constexpr int R1 = G::R1, R2 = G::R2, P = G::PS;
+  extern __shared__ float2 sm[];
+  const int slot = blockIdx.x;
+  if (!slot_runs(a.sel, slot)) return;
+  const int p = threadIdx.x, t = threadIdx.y, c = blockIdx.y * P + p, z = blockIdx.z;
+  const size_t plane = (size_t)L * a.ncont;
+  if (t < R2) {
+    float2 v[R1];
+#pragma unroll
+    for (int n1 = 0; n1 < R1; ++n1) v[n1] = make_float2(0.f, 0.f);
+    if (c < a.ncont) {
+      const float2* src = a.src + (size_t)slot * a.src_stride + c;
+      if constexpr (ADJ) {
+        const float2* k = a.k2 + z * plane + c;
+#pragma unroll
+        for (int n1 = 0; n1 < R1; ++n1) {
+          const size_t o = (size_t)(R2 * n1 + t) * a.ncont;
+          v[n1] = cmulc(__ldg(src + o), __ldg(k + o));
+        }
+      } else {
+        for (int q = 0; q < a.zchunks; ++q) {
+#pragma unroll
+          for (int n1 = 0; n1 < R1; ++n1)
+            v[n1] = cadd(v[n1], __ldg(src + q * plane + (size_t)(R2 * n1 + t) * a.ncont));
+        }
+      }
+    }
+    Dft<R1, +1>::run(v);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) sm[(k1 * R2 + t) * P + p] = k1 ? cmulc(v[k1], __ldg(a.tw + k1 * t)) : v[0];
+  }
+  __syncthreads();
+  if (c < a.ncont && t < R1) {
+    float2 u[R2];
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) u[n2] = sm[(t * R2 + n2) * P + p];
+    Dft<R2, +1, R2, R2 / 2>::run(u);
+    float2* d = a.dst + (size_t)slot * a.dst_stride + (ADJ ? z * (plane / 2) : 0) + c;
+#pragma unroll
+    for (int k2 = 0; k2 < R2 / 2; ++k2) {
+      const int y = t + R1 * k2 - (ADJ ? 0 : a.out_o);
+      if (ADJ || (y >= 0 && y < a.out_m)) d[(size_t)y * a.ncont] = u[k2];
+    }
+  }
+}
+
 // ------------------------------------------------------------------------- IX
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p));
@@ -556,6 +616,8 @@ struct PassLaunch {
   void (*fy)(const StridedParams&, int nslots, cudaStream_t);
   void (*iy)(const StridedParams&, int nslots, cudaStream_t);
   void (*z)(const ZParams&, int nslots, cudaStream_t);
+  void (*far_sum)(const FarPassParams&, int nslots, cudaStream_t);
+  void (*far_iy)(const FarPassParams&, int nslots, cudaStream_t);
   void (*ix)(const IxParams&, int nslots, cudaStream_t);
   int rows_per_cta_contig;
   int pencils_per_cta_strided;
@@ -621,6 +683,17 @@ struct PassImpl {
   }
   static void fy(const StridedParams& a, int nslots, cudaStream_t st) { strided<-1>(a, nslots, st); }
   static void iy(const StridedParams& a, int nslots, cudaStream_t st) { strided<+1>(a, nslots, st); }
+  static dim3 far_grid(const FarPassParams& a, int nslots, int nz) {
+    return dim3(nslots, (a.ncont + G::PS - 1) / G::PS, nz);
+  }
+  static void far_sum(const FarPassParams& a, int nslots, cudaStream_t st) {
+    launch_pdl((size_t)a.nz * (L / 2) * (a.ncont / 2), k_far_iy<L, false>, far_grid(a, nslots, 1), dim3(G::PS, G::T),
+               G::smem_strided, st, a);
+  }
+  static void far_iy(const FarPassParams& a, int nslots, cudaStream_t st) {
+    launch_pdl((size_t)a.nz * (L / 2) * (a.ncont / 2), k_far_iy<L, true>, far_grid(a, nslots, a.nz), dim3(G::PS, G::T),
+               G::smem_strided, st, a);
+  }
   static void z(const ZParams& a0, int nslots, cudaStream_t st) {
     ZParams a = a0;
     a.sel.nslots = nslots;
@@ -698,6 +771,8 @@ struct PassImpl {
         room(k_fxb<L>, FXB<L>::smem);
         room(k_fxb_t<L>, FXB<L>::smem);
       }
+      room(k_far_iy<L, false>, G::smem_strided);
+      room(k_far_iy<L, true>, G::smem_strided);
       room(k_ix<L>, G::smem_contig);
       room(k_ix_t<L>, G::smem_contig);
       if (e == cudaSuccess) e = set_strided_smem<-1, G::PS>((int)G::smem_strided);
@@ -724,6 +799,7 @@ struct PassImpl {
   static PassLaunch table() {
     PassLaunch t;
     t.fx = &fx; t.fy = &fy; t.iy = &iy; t.z = &z; t.ix = &ix;
+    t.far_sum = &far_sum; t.far_iy = &far_iy;
     t.rows_per_cta_contig = G::PC;
     t.pencils_per_cta_strided = G::PS;
     t.r1 = G::R1;
