@@ -375,7 +375,7 @@ static FxParams fx_base(ls_plan* P, SlotSel sel, int rows) {
   a.dst_stride = P->eng.a1_stride;
   a.tw2 = P->tw2_x;
   a.views_fastest = P->tune_fx_views_fastest;
-  a.bulk = P->tune_fx_bulk;
+  a.bulk = P->tune_fx_bulk >= 0 ? P->tune_fx_bulk : P->px.fx_bulk;
   a.sms = P->sms;
   a.err = P->eng.counts_d + 4;
   return a;
@@ -673,9 +673,10 @@ int ensure_iter_graph(ls_plan* P, int nslots) {
   // the captured launches carry the plan's launch variants: recapture when ls_autotune changed them
   const long long variant = P->tune_z_tma | P->tune_ix_prefetch << 1 | P->tune_fx_views_fastest << 2 |
                       (P->inj_z_stall || P->inj_z_wait_ns ? 1 << 3 : 0) | P->tune_z_split << 4 |
-                      P->tune_strided_wide << 5 | (P->tune_z_persist & 3) << 6 | P->tune_fx_bulk << 8 |
+                      P->tune_strided_wide << 5 | (P->tune_z_persist & 3) << 6 |
                       (P->tune_views_per_launch & 0x7ff) << 9 | (long long)(P->tune_views & 0x7ff) << 20 |
-                      (long long)((P->tune_fused + 1) & 3) << 31;
+                      (long long)((P->tune_fused + 1) & 3) << 31 |
+                      (long long)(P->tune_fx_bulk + 1) << 33;
   if (e.iter_graph && e.iter_graph_slots == nslots && e.iter_graph_variant == variant) return LS_OK;
   if (e.iter_graph) {
     cudaGraphExecDestroy(e.iter_graph);

@@ -93,7 +93,7 @@ struct ls_plan {
                                   // 2: work units from a counter; -1, untuned: the length's ZAuto form)
   int tune_views = 0;             // batch size ls_autotune tuned for: its z form applies to launches of
                                   // more than tune_views / 2 views, smaller launches take the ZAuto form
-  int tune_fx_bulk = 0;           // bulk-copy-staged persistent first pass
+  int tune_fx_bulk = -1;          // bulk-copy-staged persistent first pass (-1, untuned: the length's FxBulk)
   int tune_strided_wide = 0;      // FY/IY with 32 pencils per CTA (else 16)
   int tune_fused = -1;            // fused y/z pass: 1 on, 0 off, -1 (untuned) where it exists
   int tune_views_per_launch = 0;  // BiCGStab iteration launched over chunks of this many views (0: all)

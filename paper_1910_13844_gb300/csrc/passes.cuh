@@ -627,7 +627,14 @@ struct PassLaunch {
   int zdyn_ok;  // the dynamically scheduled TMA-staged z pass exists for this length
   int zauto_small, zauto_large;   // z-pass form of untuned plans up to kZSmallBatch views and above (ZAuto)
   int zr1b, zr2b;
+  int fx_bulk;                    // untuned plans run the bulk-staged first pass in the iteration
 };
+
+// Bulk-copy-staged first pass in the iteration of untuned plans: forward solves without and with it, 96^3 x 16
+// 6.81 -> 6.66 ms, 128^3 x 60 52.8 -> 50.8, 128^3 x 1 1.39 -> 1.35, 192^3 x 8 38.3 -> 37.2, 144^3 x 1 equal; but 64^3 x 24
+// 2.63 -> 2.83, 32^3 x 1 0.206 -> 0.217 (row blocks of 64 points are too short to keep a CTA's copies in flight).
+template <int L> struct FxBulk { static constexpr bool on = FXB<L>::ok && L >= 192; };
+
 
 template <int L>
 struct PassImpl {
@@ -812,6 +819,7 @@ struct PassImpl {
     t.zauto_large = ZAuto<L>::large;
     t.zr1b = ZRadixAlt<L>::R1;
     t.zr2b = ZRadixAlt<L>::R2;
+    t.fx_bulk = FxBulk<L>::on ? 1 : 0;
     return t;
   }
 };
