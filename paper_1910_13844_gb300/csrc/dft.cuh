@@ -127,8 +127,10 @@ struct Dft<4, DIR, NIN, NOUT> {
 template <int R> struct Split;
 template <> struct Split<6>  { static constexpr int A = 2; };
 template <> struct Split<8>  { static constexpr int A = 2; };
+template <> struct Split<9>  { static constexpr int A = 3; };
 template <> struct Split<12> { static constexpr int A = 4; };
 template <> struct Split<16> { static constexpr int A = 4; };
+template <> struct Split<18> { static constexpr int A = 6; };
 template <> struct Split<24> { static constexpr int A = 8; };
 template <> struct Split<32> { static constexpr int A = 8; };
 

@@ -42,7 +42,10 @@ struct YzParams {
   int sms;
 };
 
-// ny = RA RB on T threads per row
+// ny = RA RB on T threads per row.  RB = 2 T where it can be: a thread's loads are then pairs, and a row's are
+// contiguous (144 = 9 16 instead of 12 12 and 72 = 9 8 instead of 12 6, whose threads kept three or one and a half
+// transforms of the first stage: 144x128 planes, eight views with nx = 64, 47.7 -> 36.6 us a view; 144x96
+// 35.6 -> 28.7; 144x144, with the z split below, 58.5 -> 55.8; 72x32 5.4 -> 4.7).
 template <int NY> struct YSplit;
 template <> struct YSplit<8>   { static constexpr int RA = 4, RB = 2, T = 4; };
 template <> struct YSplit<12>  { static constexpr int RA = 4, RB = 3, T = 4; };
@@ -51,12 +54,12 @@ template <> struct YSplit<24>  { static constexpr int RA = 4, RB = 6, T = 4; };
 template <> struct YSplit<32>  { static constexpr int RA = 8, RB = 4, T = 4; };
 template <> struct YSplit<48>  { static constexpr int RA = 8, RB = 6, T = 4; };
 template <> struct YSplit<64>  { static constexpr int RA = 8, RB = 8, T = 4; };
-template <> struct YSplit<72>  { static constexpr int RA = 12, RB = 6, T = 4; };
+template <> struct YSplit<72>  { static constexpr int RA = 9, RB = 8, T = 4; };
 template <> struct YSplit<96>  { static constexpr int RA = 12, RB = 8, T = 4; };
 template <> struct YSplit<128> { static constexpr int RA = 8, RB = 16, T = 8; };
-template <> struct YSplit<144> { static constexpr int RA = 12, RB = 12, T = 4; };
+template <> struct YSplit<144> { static constexpr int RA = 9, RB = 16, T = 8; };
 template <> struct YSplit<192> { static constexpr int RA = 12, RB = 16, T = 8; };
-// 2 nz = R1 R2 (R1 even) on T threads per column
+// 2 nz = R1 R2 (R1 even) on T threads per column (288 = 16 18, not 24 12: 60 registers fewer, 96x144 35.0 -> 32.4 us)
 template <int NZ> struct ZSplit2;
 template <> struct ZSplit2<8>   { static constexpr int R1 = 4, R2 = 4, T = 4; };
 template <> struct ZSplit2<12>  { static constexpr int R1 = 4, R2 = 6, T = 4; };
@@ -68,7 +71,7 @@ template <> struct ZSplit2<64>  { static constexpr int R1 = 16, R2 = 8, T = 8; }
 template <> struct ZSplit2<72>  { static constexpr int R1 = 12, R2 = 12, T = 16; };
 template <> struct ZSplit2<96>  { static constexpr int R1 = 24, R2 = 8, T = 8; };
 template <> struct ZSplit2<128> { static constexpr int R1 = 16, R2 = 16, T = 16; };
-template <> struct ZSplit2<144> { static constexpr int R1 = 24, R2 = 12, T = 16; };
+template <> struct ZSplit2<144> { static constexpr int R1 = 16, R2 = 18, T = 16; };
 template <> struct ZSplit2<192> { static constexpr int R1 = 24, R2 = 16, T = 16; };
 
 __host__ __device__ constexpr int cdiv(int a, int b) { return (a + b - 1) / b; }
@@ -103,10 +106,10 @@ struct YZ {
   static constexpr size_t col_bytes = (size_t)2 * NY * sizeof(int);
   static constexpr size_t fixed = tile_bytes + ytab_bytes + ztab_bytes + col_bytes + misc;
   static constexpr int room = fixed < budget ? imin(16, (int)((budget - fixed) / warp_bytes)) : 0;
-  // Tensor memory, in columns: the partial outputs of a row group (2 RA floats per sub-transform), and a
+  // Tensor memory, in columns: the partial outputs of a row group (2 RA floats per sub-transform, RA made even), and a
   // lane's twiddles of the z stages and of the y stages of both parities.  Slot of a row group among those
   // of its lane quarter (the warps of a quarter are 4 apart), for w warps:
-  static constexpr int TCOL = SA * 2 * RA;
+  static constexpr int RAE = RA + RA % 2, TCOL = SA * 2 * RAE;
   static constexpr __host__ __device__ int slot(int g, int w) { return w % 4 == 0 ? g / 4 : g / w * cdiv(w, 4) + g % w / 4; }
   static constexpr int tpart(int w) { return TCOL * (w % 4 == 0 ? cdiv(NRG, 4) : cdiv(NRG, w) * cdiv(w, 4)); }
   static constexpr int TZW = S1 * 2 * R1 + S2 * 2 * R2, TYW = 4 * SA * RA + 4 * SB * RB;
@@ -139,17 +142,19 @@ struct YZ {
   static constexpr int MINB0 = imax(1, per_sm(NW));
   static constexpr int TZ1 = tpart(NW), TZ2 = TZ1 + S1 * 2 * R1, TYA = TZ1 + TZW, TYB = TYA + 4 * SA * RA;
   static constexpr bool ZT = WIDE;
-  static constexpr bool YT = ZT && pow2_at_least(TYA + TYW, 32) * MINB0 <= 512;
+  static constexpr bool YT = ZT && RA % 2 == 0 && pow2_at_least(TYA + TYW, 32) * MINB0 <= 512;
   static constexpr int TMEM = pow2_at_least(YT ? TYA + TYW : ZT ? TYA : TZ1, 32);
   static constexpr int MINB = MINB0;
   // the next half's first rows are loaded before the inverse y transform where the registers allow it
   // (at 128 a thread they would spill: 57 instead of 52 us a view at 128^3)
   static constexpr bool CROSS = 65536 / (NT * MINB) >= 160;
-  // Against FY, Z and IY as three launches, measured over all pairs of lengths with nx = 64: one view, 1.0 to
-  // 2.2 times as fast wherever the tile fits; 16M voxels in flight, 1.0 to 1.5 times, but 0.77 to 0.97 of
-  // their rate with ny = 72 or 144 and nz >= 64 (a quarter of the lanes idle in their y stages, or loads of
-  // 32 contiguous bytes), with nz = 8 and with ny = 8 and nz >= 48 (few warps).
-  static constexpr bool large_ok = !((NY == 72 || NY == 144) && NZ >= 64) && NZ != 8 && !(NY == 8 && NZ >= 48);
+  // Against FY, Z and IY as three launches, measured over all pairs of lengths with nx = 64: one view, 1.1 to
+  // 2.2 times as fast wherever the tile fits; 16M voxels in flight, 1.0 to 1.5 times, but 0.86 to 0.98 of
+  // their rate with ny = 72 and nz = 72, 128 and more, with ny = 144 and nz = 72 or 144 (a quarter to a half of
+  // the lanes idle in one of their stages, eight or nine warps an SM), with nz = 8 and with ny = 8 and nz >= 48
+  // (few warps).
+  static constexpr bool large_ok = !(NY == 72 && NZ >= 72 && NZ != 96) && !(NY == 144 && (NZ == 72 || NZ == 144)) &&
+                                   NZ != 8 && !(NY == 8 && NZ >= 48);
   static constexpr size_t smem_z = tile_bytes + col_bytes + (size_t)NW * warp_bytes;
   static constexpr size_t smem = smem_z + (YT ? 0 : ytab_bytes) + (ZT ? 0 : ztab_bytes);
 };
@@ -210,7 +215,7 @@ __device__ __forceinline__ void tmem_loaded(float2* v) {
 
 // v[a] *= exp(DIR 2 pi i a / (2 RA)), the twist of the odd half, with compile-time factors
 template <int RA, int DIR, int A = 1>
-__device__ __forceinline__ void twist(float2 (&v)[RA]) {
+__device__ __forceinline__ void twist(float2* v) {
   if constexpr (A < RA) {
     v[A] = twc<A, 2 * RA, DIR>(v[A]);
     twist<RA, DIR, A + 1>(v);
@@ -525,7 +530,7 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
           const bool has = NZ % 16 == 0 || row_a(g) < NZ;
           const int z = NZ % 16 == 0 ? row_a(g) : imin(row_a(g), NZ - 1);
           const float2* row = tile + z * PZ;
-          float2 o[SA][RA];
+          float2 o[SA][W::RAE] = {};
 #pragma unroll
           for (int s = 0; s < SA; ++s) {
             const int b = SA * TY == RB ? sub_a(s) : imin(sub_a(s), RB - 1);
@@ -534,13 +539,13 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
             Dft<RA, +1>::run(o[s]);
             if (P) twist<RA, +1>(o[s]);
             // tensor-memory accesses are warp-collective: every lane takes part, with its own values
-            const unsigned ta = tq + (unsigned)(W::slot(g, NW) * W::TCOL + s * 2 * RA);
+            const unsigned ta = tq + (unsigned)(W::slot(g, NW) * W::TCOL + s * 2 * W::RAE);
             if (P == 0) {
-              tmem_st<RA>(ta, o[s]);
+              tmem_st<W::RAE>(ta, o[s]);
             } else {
-              float2 w[RA];
-              tmem_ld<RA>(ta, w);
-              tmem_loaded<RA>(w);
+              float2 w[W::RAE];
+              tmem_ld<W::RAE>(ta, w);
+              tmem_loaded<W::RAE>(w);
 #pragma unroll
               for (int i = 0; i < RA; ++i) o[s][i] = cadd(o[s][i], w[i]);
             }

@@ -44,7 +44,7 @@ def test_operator_matches_the_oracle(ny, nz):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("shape", [(24, 24, 24), (72, 72, 16)])
+@pytest.mark.parametrize("shape", [(24, 24, 24), (72, 72, 16), (64, 144, 8), (96, 72, 8)])
 def test_many_views_take_several_planes_per_cta(shape):
     torch, ls = torch_and_lib()
     views = 70
