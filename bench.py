@@ -126,7 +126,7 @@ def source_hash(files):
     return h.hexdigest()[:16]
 
 
-Z_SOURCES = ["paper_1910_13844_gb300/csrc/zpass.cuh", "paper_1910_13844_gb300/csrc/pass_common.cuh",
+Z_SOURCES = ["paper_1910_13844_gb300/csrc/yz.cuh", "paper_1910_13844_gb300/csrc/pass_common.cuh",
              "paper_1910_13844_gb300/csrc/dft.cuh", "paper_1910_13844_gb300/csrc/common.cuh"]
 
 
@@ -152,7 +152,7 @@ def traffic_per_slot(kernel: str, field: str = "dram_bytes_per_slot"):
 
 
 def alu_roofline(opcodes, launch_ms, views_per_launch, fp32_peak, sm_count):
-    """The z pass against the FP32 pipe, with a measured denominator.
+    """The fused y/z pass against the FP32 pipe, with a measured denominator.
 
     opcodes: ncu's warp-level counts per view of the pass's FP32 instructions (FADD2, FFMA, FMUL);
     fp32_peak: lane operations per second of each kind measured on this GPU by ls_fp32_peak.  The
@@ -165,12 +165,55 @@ def alu_roofline(opcodes, launch_ms, views_per_launch, fp32_peak, sm_count):
     floor_s = sum(lanes[k] * opcodes[k] / fp32_peak[k] for k in lanes)
     achieved = ops * views_per_launch / (launch_ms / 1e3) / 1e12
     peak = ops / floor_s / 1e12
-    return {"kernel": "k_zw", "bound": "alu", "achieved": round(achieved, 2), "peak": round(peak, 2),
+    return {"kernel": "k_yz", "bound": "alu", "achieved": round(achieved, 2), "peak": round(peak, 2),
             "unit": "T FP32 lane-ops/s", "frac": round(achieved / peak, 4), "ops_per_view": int(ops),
             "peak_source": "measured: ls_fp32_peak (FFMA, FMUL, packed FADD2 microkernels) weighted by the "
                            "pass's ncu opcode mix", "fp32_peak_lane_ops_per_s": {k: round(v / 1e12, 2) for k, v in
                                                                                 fp32_peak.items()},
             "sm_count": sm_count}
+
+
+def fused_yz(prof):
+    """Whether profiled plain applications of the operator ran FY, Z and IY as the one fused launch: the profiler
+    then counts it once for each of the three and divides its time 1 : 2 : 1."""
+    fy, z, iy = (prof[k][0] for k in ("fy", "z", "iy"))
+    return z > 0 and abs(fy - iy) <= 1e-6 * z and abs(z - 2 * fy) <= 1e-6 * z
+
+
+def split_fused(prof):
+    """prof with the fused launches under "yz"; what is left under FY and IY are those of the far-field operators."""
+    out = {k: tuple(v) for k, v in prof.items() if k != "z"}
+    ms, launches, slots, active = prof["z"]
+    out["yz"] = (2 * ms, launches, slots, active)
+    for k in ("fy", "iy"):
+        v = prof[k]
+        out[k] = (max(v[0] - ms / 2, 0.0), v[1] - launches, v[2] - slots, v[3] - active)
+    return out
+
+
+def operator_passes(prof, shape):
+    """name -> (bytes per view, bytes per launch, ms, launches, active views) of the passes of the operator:
+    the plain matvec's traffic, each pass reading its input and writing its output once."""
+    nz, ny, nx = shape
+    N = nx * ny * nz
+    if "yz" in prof:
+        green = 8 * (nx + 1) * (ny + 1) * 2 * nz
+        return {"fx": (28 * N, 0) + pass_of(prof, "fx"), "yz": (32 * N, green) + pass_of(prof, "yz"),
+                "ix": (32 * N, 0) + pass_of(prof, "ix")}
+    octant = 8 * (nx + 1) * (ny + 1) * (nz + 1)
+    per_view = {"fx": 28 * N, "fy": 48 * N, "z": 64 * N, "iy": 48 * N, "ix": 32 * N}
+    return {k: (b, octant if k == "z" else 0) + pass_of(prof, k) for k, b in per_view.items()}
+
+
+def pass_of(prof, k):
+    return prof[k][0], prof[k][1], prof[k][3]
+
+
+def rates(passes):
+    """({pass: GB/s}, total bytes, total ms) of operator_passes."""
+    total = {k: b * active + per_launch * n for k, (b, per_launch, _, n, active) in passes.items()}
+    gbs = {k: round(total[k] / (v[2] / 1e3) / 1e9, 1) for k, v in passes.items() if v[2] > 0}
+    return gbs, sum(total.values()), sum(v[2] for v in passes.values())
 
 
 def dist_env():
@@ -356,40 +399,25 @@ def run_gpu(args):
     value = ws * solves_per_step / (ms_step / 1e3)
     e2e_value = ws * solves_per_step / (ms_e2e_step / 1e3)
 
-    # roofline of the dominant kernel (the z pass: FFT, Green multiply, IFFT); bytes counted for the
-    # slots that actually ran (converged views are masked off inside the launches)
+    # roofline of the dominant kernel (the fused y/z pass, or the z pass of the three: FFT, Green multiply,
+    # IFFT); bytes counted for the slots that actually ran (converged views are masked off inside the launches)
     N = shape[0] * shape[1] * shape[2]
-    nz, ny, nx = shape
-    octant = 8 * (nx + 1) * (ny + 1) * (nz + 1)            # Green spectrum octant, read once per launch
-    pass_bytes = {"fx": 28 * N, "fy": 48 * N, "z": 64 * N, "iy": 48 * N, "ix": 32 * N}   # plain-matvec model
-    pass_gbs = {}
-    mv_bytes = mv_ms = 0.0
-    for k, b in pass_bytes.items():
-        ms_k, launches_k, _, active_k = prof[k]
-        byt = b * active_k + (octant * launches_k if k == "z" else 0)
-        if ms_k > 0:
-            pass_gbs[k] = round(byt / (ms_k / 1e3) / 1e9, 1)
-        mv_bytes += byt
-        mv_ms += ms_k
-    iso_gbs = {}
-    iso_bytes = iso_ms = 0.0
-    for k, b in pass_bytes.items():
-        ms_k, launches_k, _, active_k = iso[k]
-        byt = b * active_k + (octant * launches_k if k == "z" else 0)
-        if ms_k > 0:
-            iso_gbs[k] = round(byt / (ms_k / 1e3) / 1e9, 1)
-        iso_bytes += byt
-        iso_ms += ms_k
+    fused = fused_yz(iso)
+    if fused:
+        prof, iso = split_fused(prof), split_fused(iso)
+    passes = operator_passes(prof, shape)
+    pass_gbs, mv_bytes, mv_ms = rates(passes)
+    iso_gbs, iso_bytes, iso_ms = rates(operator_passes(iso, shape))
     # BiCGStab update x += alpha p + omega s, r = s - omega t, <rh, r>: reads p, s, t, rh, x, writes x, r
     upd_ms, _, _, upd_active = prof.get("update", (0.0, 0, 0, 0))
     update_gbs = round(56 * N * upd_active / (upd_ms / 1e3) / 1e9, 1) if upd_ms > 0 else None
-    z_ms, z_launches, _, z_active = prof["z"]
+    z_bytes, z_green, z_ms, z_launches, z_active = passes["yz" if fused else "z"]
     active_per_launch = z_active / max(z_launches, 1)
-    bytes_per_launch = 64 * N * active_per_launch + octant
+    bytes_per_launch = z_bytes * active_per_launch + z_green
     z_ms_launch = z_ms / max(z_launches, 1)
     achieved = bytes_per_launch / (z_ms_launch / 1e3) / 1e9
     peak, peak_kind = measured_peaks()
-    tr = traffic_per_slot("z_pass")
+    tr = traffic_per_slot("yz_pass") if fused else None
     dominant = max((k for k in prof if k != "other"), key=lambda k: prof[k][0])
     total_kernel_ms = sum(v[0] for v in prof.values())
     launches = int(sum(v[1] for v in prof.values()))
@@ -421,34 +449,36 @@ def run_gpu(args):
                          if tune else "off (defaults)"),
         },
         "roofline": {
-            "kernel": "k_z (z-pencil FFT, Green multiply, inverse FFT, crop)",
+            "kernel": ("k_yz (y FFT, z FFT, Green multiply, both inverses, crop; bound by the FP32 and shared-memory pipes)"
+                       if fused else "k_z (z-pencil FFT, Green multiply, inverse FFT, crop)"),
             "bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
             "frac": round(achieved / peak, 4), "peak_source": peak_kind,
             "traffic": (round(tr * active_per_launch) if tr is not None else None),
             "algorithmic_bytes_per_launch": int(bytes_per_launch),
             "launch_ms": round(z_ms_launch, 4), "active_views_per_launch": round(active_per_launch, 2),
         },
-        "roofline_alu": alu_roofline(opcodes_per_slot("z_pass"), z_ms_launch, active_per_launch, fp32_peak,
+        "roofline_alu": alu_roofline(opcodes_per_slot("yz_pass") if fused else None, z_ms_launch, active_per_launch, fp32_peak,
                                      torch.cuda.get_device_properties(dev).multi_processor_count),
         "matvec": {
             "gbs": round(mv_bytes / (mv_ms / 1e3) / 1e9, 1) if mv_ms else None,
             "frac_hbm": round(mv_bytes / (mv_ms / 1e3) / 1e9 / peak, 4) if mv_ms else None,
-            "us_per_view": round(1e3 * mv_ms / max(prof["z"][3], 1), 2),
+            "us_per_view": round(1e3 * mv_ms / max(z_active, 1), 2),
             "pass_gbs": pass_gbs,
-            "bytes_model": "plain matvec per view: F-x 28N, F-y 48N, Z 64N + Ghat octant per launch, I-y 48N, "
-                           "I-x 32N bytes (the fused BiCGStab prologue/epilogue traffic is not counted)",
+            "bytes_model": ("plain matvec per view: F-x 28N, fused y/z 32N + the Green values per launch, I-x 32N bytes"
+                            if fused else "plain matvec per view: F-x 28N, F-y 48N, Z 64N + Ghat octant per launch, I-y 48N, "
+                                          "I-x 32N bytes") + " (the fused BiCGStab prologue/epilogue traffic is not counted)",
         },
         "matvec_all_views_active": {
             "gbs": round(iso_bytes / (iso_ms / 1e3) / 1e9, 1) if iso_ms else None,
             "frac_hbm": round(iso_bytes / (iso_ms / 1e3) / 1e9 / peak, 4) if iso_ms else None,
-            "us_per_view": round(1e3 * iso_ms / max(iso["z"][3], 1), 2),
+            "us_per_view": round(1e3 * iso_ms / max(iso["yz" if fused else "z"][3], 1), 2),
             "pass_gbs": iso_gbs,
-            "how": f"ls_matvec_batch over all {Q} views, 5 launches per pass, same byte model",
+            "how": f"ls_matvec_batch over all {Q} views, 5 repeats, same byte model",
         },
         "cufft_matvec": {
             "us_per_view": round(cufft_us, 2) if cufft_us else None,
-            "ours_us_per_view": round(1e3 * iso_ms / max(iso["z"][3], 1), 2),
-            "speedup": round(cufft_us / (1e3 * iso_ms / max(iso["z"][3], 1)), 3) if cufft_us and iso_ms else None,
+            "ours_us_per_view": round(1e3 * iso_ms / max(iso["yz" if fused else "z"][3], 1), 2),
+            "speedup": round(cufft_us / (1e3 * iso_ms / max(iso["yz" if fused else "z"][3], 1)), 3) if cufft_us and iso_ms else None,
             "max_rel_diff": cufft_diff,
             "how": "torch.fft (cuFFT) C2C 3-D on the zero-padded f x, full Green spectrum multiply, inverse, "
                    "crop, subtract; 10 views per batched transform; timed comparison only",
@@ -775,8 +805,6 @@ def run_bead_mode(args):
         dnd = torch.from_numpy(ph.sphere(shape, radius / h, dn_bead).astype(np.float32)).cuda()
         f = torch.empty_like(dnd)
         ls.ls_scattering_potential(dnd, eta_b, kb, f)
-        N = n ** 3
-        octant = 8 * (n + 1) ** 3
         for Q in (1, 16):
             kvec = np.array([[0.0, 0.0, kb]]) if Q == 1 else ph.cone_directions(Q, NA, eta_b) * kb
             tune = plan.autotune(Q, f)
@@ -802,18 +830,18 @@ def run_bead_mode(args):
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1) / reps
             ls.ls_profile(plan.handle, True)
-            solve()
+            ls.ls_forward(plan.handle, f, uin, u)
             torch.cuda.synchronize()
             prof = ls.ls_profile(plan.handle, False)
-            z_ms, z_launches, _, z_active = prof["z"]
-            z_gbs = (64 * N * z_active + octant * z_launches) / (z_ms / 1e3) / 1e9 if z_ms else None
+            fused = fused_yz(prof)
+            z_gbs = rates(operator_passes(split_fused(prof) if fused else prof, (n, n, n)))[0].get("yz" if fused else "z")
             its = [s["iterations"] for _, st in stats[-reps:] for s in st]
             out[f"{n}^3_{Q}_views"] = {
                 "solves_per_s": round(Q / (ms / 1e3), 2), "ms_per_batch": round(ms, 3),
                 "mean_iterations": float(np.mean(its)),
                 "worst_status": int(max(c for c, _ in stats)),
                 "z_pass_gbs": round(z_gbs, 1) if z_gbs else None,
-                "z_kernel": ("k_zg (TMA-staged column groups)" if tune["z_tma"] else "k_z (cp.async staging)")
+                "z_kernel": "k_yz (fused y/z pass)" if fused else ("k_zg (TMA-staged column groups)" if tune["z_tma"] else "k_z (cp.async staging)")
                 if 2 * n in (144, 288) else ("k_zw" if tune["z_tma"] else "k_z (cp.async staging)"),
                 "autotune": {k: tune[k] for k in ("z_tma", "z_split", "z_persist", "strided_wide", "ix_prefetch", "fx_views_fastest", "fx_bulk",
                                                   "views_per_launch", "check_every", "use_graphs")},

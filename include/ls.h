@@ -185,6 +185,8 @@ int ls_matvec_noalloc(const ls_plan* plan, const float* f, const ls_c64* x, ls_c
  * solver's workspace (no caller buffer, no copies).  u_out[q] (N) and
  * far[q] (my*mx) may each be NULL (u_out == NULL: fields not returned;
  * far == NULL: far field skipped).  stats: host array of n_views or NULL.
+ * The kernels read and write these vectors where they are; vectors that overlap one
+ * another (u_out[q] == u_in[q]) go through the workspace.
  * Returns LS_OK, LS_NOT_CONVERGED, LS_BREAKDOWN or LS_TIMEOUT (worst view), or an error;
  * LS_ECUDA also when a z-pass wait on its own TMA copy gave up (bounded, one second). */
 int ls_forward(ls_plan* plan, const float* f, int n_views, const ls_c64* const* u_in,
@@ -241,8 +243,9 @@ int ls_prox_hs(const ls_grid* grid, const float* z, float* x, double lam, int it
  * potential f (device, N floats), one knob after the other, and keeps the fastest in the plan (the
  * plan's check_every / use_graphs options are overwritten).  If the environment variable
  * LS_AUTOTUNE_CACHE names a file, a result for the same device, grid and view count is read from it
- * instead of timing, and new results are appended to it.  The z-pass form chosen applies to launches
- * of more than n_views / 2 views; smaller batches on the same plan keep the per-length default form
+ * instead of timing, and new results are appended to it (a line's last field says whether FY, Z and
+ * IY run as one fused pass; lines without it run the three).  The z-pass form chosen, fused or not,
+ * applies to launches of more than n_views / 2 views; smaller batches on the same plan keep the per-length default form
  * (the fastest form depends on the batch size).  Synchronous; uses the plan's workspace (its
  * contents are overwritten).  out may be NULL.  No counterpart in the paper. */
 int ls_autotune(ls_plan* plan, int n_views, const float* f, ls_tune* out, void* cuda_stream);
@@ -332,7 +335,9 @@ void ls_server_destroy(ls_server* srv);
 /* ---------------------------------------------------------------- profiling */
 
 /* Kernel kinds timed by ls_profile (the five FFT passes of one operator
- * application, the BiCGStab update and scalar steps, far-field kernels). */
+ * application, the BiCGStab update and scalar steps, far-field kernels).
+ * Where FY, Z and IY run as one fused launch, it counts once for each of the
+ * three, and its time is divided between them 1 : 2 : 1. */
 enum ls_kernel_kind {
   LS_K_FX = 0, LS_K_FY = 1, LS_K_Z = 2, LS_K_IY = 3, LS_K_IX = 4,
   LS_K_UPDATE = 5, LS_K_SCALAR = 6, LS_K_FAR = 7, LS_K_OTHER = 8, LS_K_COUNT = 9
