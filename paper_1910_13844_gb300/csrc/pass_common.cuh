@@ -195,16 +195,35 @@ template <> struct Radix<256> { static constexpr int R1 = 16, R2 = 16; };
 template <> struct Radix<288> { static constexpr int R1 = 12, R2 = 24; };
 template <> struct Radix<384> { static constexpr int R1 = 16, R2 = 24; };
 
+// rows per CTA, contiguous passes with t threads per row: the largest count <= 256 / t that makes whole warps
+__host__ __device__ constexpr int rows_per_cta(int t) {
+  return (t * (256 / t)) % 32 == 0 ? 256 / t : (t * (192 / t)) % 32 == 0 ? 192 / t : 32;
+}
+
+// Threads per row and rows per CTA of the plain first pass.  One thread per sub-transform of the longer stage;
+// for 128 = 16 8 of the shorter one (eight threads that make two 8-point transforms each), since half of 16 would
+// have nothing to load: the pass in 64^3 x 24 operators 2.02 -> 1.64 us a view (60 views 1.82 -> 1.40), with 16 rows a
+// CTA; with 32 it was slower in the iteration's modes.  The other unequal splits idle less, and their CTAs with
+// twice the rows were 5-10% slower.
+template <int L>
+struct FxRows {
+  static constexpr int T = imax(Radix<L>::R1, Radix<L>::R2), P = rows_per_cta(T);
+};
+template <>
+struct FxRows<128> { static constexpr int T = 8, P = 16; };
+
 template <int L>
 struct Geo {
   static constexpr int R1 = Radix<L>::R1, R2 = Radix<L>::R2;
   static constexpr int T = imax(R1, R2);
-  // rows per CTA, contiguous passes: the largest count <= 256/T that makes whole warps
-  static constexpr int PC = (T * (256 / T)) % 32 == 0 ? 256 / T : (T * (192 / T)) % 32 == 0 ? 192 / T : 32;
+  static constexpr int PC = rows_per_cta(T);
   static constexpr int PS = 16;                              // pencils per CTA, strided passes
   static constexpr int ZMINB = (T * PS > 256) ? 1 : 2;   // resident CTAs per SM asked of the z pass
   static constexpr int SROW = R2 + 1;                        // padded row of the contiguous exchange
   static constexpr int XROW = R1 * SROW | 1;                 // a row's exchange block, odd: PC rows on disjoint banks
+  // threads per row and rows per CTA of the plain first pass
+  static constexpr int TF = FxRows<L>::T, PF = FxRows<L>::P;
+  static constexpr size_t smem_fx = (size_t)PF * XROW * sizeof(float2);
   static constexpr size_t smem_contig = (size_t)PC * XROW * sizeof(float2);
   static constexpr size_t smem_strided = (size_t)L * PS * sizeof(float2);
   static constexpr size_t smem_z = (size_t)(2 * L + L) * PS * sizeof(float2);   // exchange + Ghat + 2 staging halves

@@ -62,27 +62,33 @@ __device__ __forceinline__ void block_sum_store(const float (&acc)[NV], double* 
 // kx, [row][2nx].  TR: lanes along the CTA's PC rows, [kx][rows]; the rows of a block are consecutive y
 // (and z) positions, so PC lanes write one contiguous run.  The odd pitch of a row's exchange block keeps
 // both directions free of bank conflicts.
-template <int L, bool TR>
+// TT threads per row, PC rows per CTA.
+template <int L, bool TR, int TT, int PC>
 __device__ __forceinline__ void fx_store(const FxParams& a, const float2* sm, int slot, int rb) {
   using G = Geo<L>;
-  constexpr int R1 = G::R1, R2 = G::R2, PC = G::PC;
-  const int tid = threadIdx.y * G::T + threadIdx.x;
-  const int p = TR ? tid % PC : threadIdx.y, t = TR ? tid / PC : threadIdx.x;
+  constexpr int R1 = G::R1, R2 = G::R2;
+  const int tid = threadIdx.y * TT + threadIdx.x;
+  const int p = TR ? tid % PC : threadIdx.y, t0 = TR ? tid / PC : threadIdx.x;
   const int row = rb * PC + p;
-  if (row >= a.rows || t >= R1) return;
-  const float2* S = sm + (size_t)p * G::XROW + t * G::SROW;
-  float2 u[R2];
-#pragma unroll
-  for (int n2 = 0; n2 < R2; ++n2) u[n2] = S[n2];
-  Dft<R2, -1>::run(u);
+  if (row >= a.rows) return;
   float2* d = a.dst + (size_t)slot * a.dst_stride + (TR ? (size_t)row : (size_t)row * L);
 #pragma unroll
-  for (int k2 = 0; k2 < R2; ++k2) {
-    const int kx = t + R1 * k2;
-    const size_t o = TR ? (size_t)kx * a.rows : (size_t)kx;
-    if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, o + (TR ? (size_t)row : (size_t)row * L), (size_t)a.rows * L,
-                                  a.dst_stride), BS_FX_DST))
-      d[o] = u[k2];
+  for (int t1 = 0; t1 < R1; t1 += TT) {
+    const int t = t0 + t1;
+    if (t >= R1) break;
+    const float2* S = sm + (size_t)p * G::XROW + t * G::SROW;
+    float2 u[R2];
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) u[n2] = S[n2];
+    Dft<R2, -1>::run(u);
+#pragma unroll
+    for (int k2 = 0; k2 < R2; ++k2) {
+      const int kx = t + R1 * k2;
+      const size_t o = TR ? (size_t)kx * a.rows : (size_t)kx;
+      if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, o + (TR ? (size_t)row : (size_t)row * L), (size_t)a.rows * L,
+                                    a.dst_stride), BS_FX_DST))
+        d[o] = u[k2];
+    }
   }
 }
 
@@ -102,7 +108,8 @@ __device__ __forceinline__ void fx_body(const FxParams& a) {
   count_run_if(a.sel, rb == 0);
   const int t = threadIdx.x, p = threadIdx.y;
   const int nx = L / 2;
-  const int row = rb * G::PC + p;
+  static_assert(G::TF >= R2, "one first-stage transform per thread");
+  const int row = rb * G::PF + p;
   const bool valid = row < a.rows;
   const size_t voff = (size_t)slot * a.vstride + (size_t)row * nx;
   const float* f = slot_f(a.sel, slot);
@@ -161,13 +168,16 @@ __device__ __forceinline__ void fx_body(const FxParams& a) {
     for (int k1 = 0; k1 < R1; ++k1) S[k1 * G::SROW + t] = v[k1];
   }
   __syncthreads();
-  fx_store<L, TR>(a, sm, slot, rb);
+  fx_store<L, TR, G::TF, G::PF>(a, sm, slot, rb);
 }
 
+// Six CTAs of 192-256 threads an SM; ten of 128 (nx = 64; with twelve, 40 registers, the three-vector modes spill:
+// 64^3 x 24 solve 2.73 ms, ten 2.64, 16 threads a row 2.70; 128x128x64 x 16 8.15, 8.08, 8.42).
+template <int L> struct FxCtas { static constexpr int MINB = Geo<L>::TF * Geo<L>::PF < 192 ? 10 : 6; };
 template <int L>
-__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 6) k_fx(FxParams a) { fx_body<L, false>(a); }
+__global__ void __launch_bounds__(Geo<L>::TF * Geo<L>::PF, FxCtas<L>::MINB) k_fx(FxParams a) { fx_body<L, false>(a); }
 template <int L>
-__global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PC, 6) k_fx_t(FxParams a) { fx_body<L, true>(a); }
+__global__ void __launch_bounds__(Geo<L>::TF * Geo<L>::PF, FxCtas<L>::MINB) k_fx_t(FxParams a) { fx_body<L, true>(a); }
 
 // ------------------------------------------------------------------------- FX (bulk-copy staged)
 // The same pass with the rows of every input vector staged in shared memory by bulk copies
@@ -328,7 +338,7 @@ __device__ __forceinline__ void fxb_body(const FxParams& a) {
     __syncthreads();
     // every thread has read its inputs from stage s: refill it with the item NSTG ahead
     if (tid == 0 && m + NSTG < nmine) issue(m + NSTG, s);
-    fx_store<L, TR>(a, S0, slot, rb);
+    fx_store<L, TR, G::T, G::PC>(a, S0, slot, rb);
     __syncthreads();   // the exchange area is free for the next item
   }
   (void)NT;
@@ -655,12 +665,12 @@ struct PassImpl {
         return;
       }
     }
-    const unsigned rbs = (unsigned)((a.rows + G::PC - 1) / G::PC);
-    dim3 blk(G::T, G::PC), grd = a.views_fastest ? dim3(nslots, rbs) : dim3(rbs, nslots);
+    const unsigned rbs = (unsigned)((a.rows + G::PF - 1) / G::PF);
+    dim3 blk(G::TF, G::PF), grd = a.views_fastest ? dim3(nslots, rbs) : dim3(rbs, nslots);
     FxParams b = a;
     b.sel.nslots = nslots;
-    if (a.transposed) launch_pdl((size_t)a.rows * (L / 2), k_fx_t<L>, grd, blk, G::smem_contig, st, b);
-    else launch_pdl((size_t)a.rows * (L / 2), k_fx<L>, grd, blk, G::smem_contig, st, b);
+    if (a.transposed) launch_pdl((size_t)a.rows * (L / 2), k_fx_t<L>, grd, blk, G::smem_fx, st, b);
+    else launch_pdl((size_t)a.rows * (L / 2), k_fx<L>, grd, blk, G::smem_fx, st, b);
   }
   static void ix(const IxParams& a0, int nslots, cudaStream_t st) {
     IxParams a = a0;
@@ -772,8 +782,8 @@ struct PassImpl {
       auto room = [&](auto kernel, size_t bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
       };
-      room(k_fx<L>, G::smem_contig);
-      room(k_fx_t<L>, G::smem_contig);
+      room(k_fx<L>, G::smem_fx);
+      room(k_fx_t<L>, G::smem_fx);
       if constexpr (FXB<L>::ok) {
         room(k_fxb<L>, FXB<L>::smem);
         room(k_fxb_t<L>, FXB<L>::smem);
