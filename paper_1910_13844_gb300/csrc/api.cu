@@ -1284,20 +1284,22 @@ int ls_matvec_batch(ls_plan* P, const float* f, int n_views, const ls_c64* const
     if (x[q] != y[q]) io.add(x[q], e.N * sizeof(float2), false);
   }
   const bool direct = io.disjoint();
-  // states from pageable memory: the copy is taken before the call returns (the call does not synchronise)
-  std::vector<SlotDev> slots(n_views);
-  for (int q = 0; q < n_views; ++q) {
-    slot_defaults(P, slots[q], q, f, adjoint ? 1 : 0);
-    slots[q].flags = SLOT_AUX;
-    slots[q].xo = e.vptr(V_R, q);
-    if (direct) {
-      slots[q].x = (const float2*)x[q];
-      slots[q].xo = (float2*)y[q];
-    } else {
-      LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), x[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+  // the call does not synchronise and may be captured: the slot states go out as kernel arguments
+  OperatorSlots s;
+  s.f = f;
+  s.adjoint = adjoint ? 1 : 0;
+  for (int q0 = 0; q0 < n_views; q0 += OperatorSlots::kMax) {
+    s.slots = e.slots_d + q0;
+    s.n = std::min(n_views - q0, OperatorSlots::kMax);
+    for (int k = 0; k < s.n; ++k) {
+      const int q = q0 + k;
+      s.x[k] = direct ? (const float2*)x[q] : e.vptr(V_X, q);
+      s.xo[k] = direct ? (float2*)y[q] : e.vptr(V_R, q);
+      if (!direct)
+        LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), x[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
     }
+    launch_operator_slots(s, e.N, st);
   }
-  LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, slots.data(), (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
   SlotSel sel = sel_slots(P, SLOT_AUX);
   FxParams fx = fx_base(P, sel, P->ny * P->nz);
   fx.mode = FX_F_TIMES;

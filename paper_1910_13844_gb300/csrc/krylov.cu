@@ -70,6 +70,20 @@ __device__ __forceinline__ bool zfinite(double2 a) { return isfinite(a.x) && isf
 // Relative breakdown threshold of BiCGStab's two inner products (the paper gives none).
 constexpr double kBreakdownRel = 1e-30;
 
+// One thread per slot: the state that the passes of an operator call read
+__global__ void __launch_bounds__(OperatorSlots::kMax) k_operator_slots(const __grid_constant__ OperatorSlots a) {
+  pdl_begin();
+  const int q = threadIdx.x;
+  if (q >= a.n) return;
+  SlotDev s = {};
+  s.f = a.f;
+  s.x = a.x[q];
+  s.xo = a.xo[q];
+  s.flags = SLOT_AUX;
+  s.adjoint = a.adjoint;
+  a.slots[q] = s;
+}
+
 // One block per slot: sums the partials of the preceding kernel in a fixed
 // order (float64), then thread 0 advances the slot's BiCGStab state.
 __global__ void __launch_bounds__(256) k_scalar(ScalarParams a) {
@@ -320,6 +334,9 @@ __global__ void __launch_bounds__(256) k_inner(ResidualParams a) {
 }
 
 // ------------------------------------------------------------------ launchers
+void launch_operator_slots(const OperatorSlots& a, size_t voxels, cudaStream_t st) {
+  launch_pdl(voxels, k_operator_slots, 1, OperatorSlots::kMax, 0, st, a);
+}
 void launch_update(const UpdParams& a0, int nblocks, int nslots, cudaStream_t st) {
   UpdParams a = a0;
   a.sel.nslots = nslots;

@@ -29,6 +29,18 @@ struct ScalarParams {
   size_t n;                 // voxels per slot
 };
 
+// States of the slots of one operator call: each reads x and writes xo.  The vectors come by value, so that the
+// launch holds all it needs: an upload from host memory would be repeated from there by a captured graph.
+struct OperatorSlots {
+  static constexpr int kMax = 128;   // views per launch (2 KB of parameters)
+  SlotDev* slots;           // of the launch's first view
+  int n;
+  const float* f;
+  int adjoint;
+  const float2* x[kMax];
+  float2* xo[kMax];
+};
+
 struct PlaneWaveParams {
   int nx, ny, nz;
   double h;
@@ -61,6 +73,7 @@ struct ResidualParams {
   double* partials;           // [view][nblocks][4]
 };
 
+void launch_operator_slots(const OperatorSlots& a, size_t voxels, cudaStream_t st);
 void launch_update(const UpdParams& a, int nblocks, int nslots, cudaStream_t st);
 void launch_scalar(const ScalarParams& a, int nslots, cudaStream_t st);
 void launch_zero_shadow(const SlotDev* slots, int slot, float2* rh, size_t n, cudaStream_t st);
