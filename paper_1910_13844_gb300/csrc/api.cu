@@ -891,11 +891,7 @@ static int pupil_on_far(ls_plan* P, int n, ls_c64* const* far, cudaStream_t st) 
   Engine& e = P->eng;
   std::vector<const void*> src(n);
   for (int q = 0; q < n; ++q) src[q] = e.far + (size_t)q * P->mx * P->my;
-  int rc = engine_upload_ptrs(P, 2, src.data(), n, st);
-  if (rc == LS_OK) rc = engine_upload_ptrs(P, 3, (const void* const*)far, n, st);
-  if (rc) return rc;
-  return apply_pupil_views(P, n, (const float2* const*)engine_ptr_table(P, 2), (float2* const*)engine_ptr_table(P, 3),
-                           0, e.a1, st);
+  return apply_pupil_views(P, n, src.data(), (void* const*)far, 0, e.a1, n, st);
 }
 
 // Uploads the table (1) of the residuals that G~^H is applied to: r_q, or P^H r_q in the engine's detector
@@ -903,13 +899,11 @@ static int pupil_on_far(ls_plan* P, int n, ls_c64* const* far, cudaStream_t st) 
 static int pupil_adjoint_residuals(ls_plan* P, int n, const ls_c64* const* r, cudaStream_t st) {
   if (!P->pupil_h) return engine_upload_ptrs(P, 1, (const void* const*)r, n, st);
   Engine& e = P->eng;
-  std::vector<const void*> dst(n);
+  std::vector<void*> dst(n);
   for (int q = 0; q < n; ++q) dst[q] = e.far + (size_t)q * P->mx * P->my;
-  int rc = engine_upload_ptrs(P, 3, (const void* const*)r, n, st);
-  if (rc == LS_OK) rc = engine_upload_ptrs(P, 1, dst.data(), n, st);
+  const int rc = engine_upload_ptrs(P, 1, dst.data(), n, st);
   if (rc) return rc;
-  return apply_pupil_views(P, n, (const float2* const*)engine_ptr_table(P, 3), (float2* const*)engine_ptr_table(P, 1),
-                           1, e.a1, st);
+  return apply_pupil_views(P, n, (const void* const*)r, dst.data(), 1, e.a1, n, st);
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }

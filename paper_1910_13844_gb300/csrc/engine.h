@@ -144,10 +144,10 @@ ls_plan* plan_clone_shared(const ls_plan* P);
 int tune_matvec(ls_plan* P, const float* f, int n, cudaStream_t st);
 // a forward solve of slots [0, n) from the right-hand sides already in V_B (x0 = b), for the autotuner
 int tune_forward(ls_plan* P, const float* f, int n, cudaStream_t st);
-// out[q] = P in[q] (adjoint: P^H in[q]) for n detector fields (device tables of their pointers; in may be out);
-// scratch holds pupil_scratch_bytes(P, n)
-int apply_pupil_views(ls_plan* P, int n, const float2* const* in, float2* const* out, int adjoint, void* scratch,
-                      cudaStream_t st);
+// out[q] = P in[q] (adjoint: P^H in[q]) for n detector fields (host arrays of device pointers; in[q] may be out[q]);
+// scratch holds pupil_scratch_bytes(P, scratch_views), scratch_views >= 1
+int apply_pupil_views(ls_plan* P, int n, const void* const* in, void* const* out, int adjoint, void* scratch,
+                      int scratch_views, cudaStream_t st);
 size_t pupil_scratch_bytes(const ls_plan* P, int n);
 
 // ls_matvec_noalloc set-up (noalloc.cu): the device address of the static scratch array on the

@@ -8,7 +8,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <vector>
 
 #include "engine.h"
 #include "fft64.cuh"
@@ -89,7 +88,7 @@ __global__ void k_pupil_transfer(int Mx, int My, double h, double kb, double kcu
   }
 }
 
-// The pupil operator P y = crop(F^{-1}(H F(pad y))) on the 2my x 2mx padded detector, for all views of a call in
+// The pupil operator P y = crop(F^{-1}(H F(pad y))) on the 2my x 2mx padded detector, for up to 64 views in
 // three launches over scratch planes [view][my][2mx] in float64: rows are padded and transformed, columns
 // padded, transformed, multiplied by H and transformed back, rows transformed back and cropped.  Rows that
 // are zero or cropped away are never touched.  Bound by the float64 pipe: 12 us a view at 72 x 72 with 20 views; one
@@ -98,19 +97,27 @@ __global__ void k_pupil_transfer(int Mx, int My, double h, double kb, double kcu
 // CTA's columns, whose elements lie next to one another in shared memory.
 constexpr int kPupilThreads = 256;
 
+// Detector fields of one launch.  They come by value, so that the launch holds all it needs: an upload from host
+// memory would be repeated from there by a captured graph.
+struct PupilViews {
+  static constexpr int kMax = 64;
+  const float2* in[kMax];
+  float2* out[kMax];
+};
+
 // out[v][y][:] = F(pad in[v][y][:]); grid (row blocks, views), `per` rows per CTA
-__global__ void __launch_bounds__(kPupilThreads) k_pupil_rows(const float2* const* in, int mx, int my, int per,
-                                                              double2* out, const double2* tw) {
+__global__ void __launch_bounds__(kPupilThreads) k_pupil_rows(const __grid_constant__ PupilViews v, int mx, int my,
+                                                              int per, double2* out, const double2* tw) {
   extern __shared__ double2 pb[];
   const int M = 2 * mx, nt = kPupilThreads / per, g = threadIdx.x / nt, t = threadIdx.x % nt;
   const int y = blockIdx.x * per + g;
   const bool has = g < per && y < my;
   double2* b = pb + (size_t)g * 2 * M;
-  const float2* src = in[blockIdx.y] + (size_t)y * mx;
+  const float2* src = v.in[blockIdx.y] + (size_t)y * mx;
   if (g < per)
     for (int i = t; i < M; i += nt) {
-      const float2 v = has && i < mx ? src[i] : make_float2(0.f, 0.f);
-      b[i] = make_double2(v.x, v.y);
+      const float2 s = has && i < mx ? src[i] : make_float2(0.f, 0.f);
+      b[i] = make_double2(s.x, s.y);
     }
   __syncthreads();
   // idle threads (g == per where per does not divide the block) run no butterfly
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(kPupilThreads) k_pupil_cols(double2* plane, in
 
 // out[v][y][:] = crop F^{-1}(plane[v][y][:]), rounded to complex64
 __global__ void __launch_bounds__(kPupilThreads) k_pupil_out(const double2* plane, int mx, int my, int per,
-                                                             float2* const* out, const double2* tw) {
+                                                             const __grid_constant__ PupilViews v, const double2* tw) {
   extern __shared__ double2 pb[];
   const int M = 2 * mx, nt = kPupilThreads / per, g = threadIdx.x / nt, t = threadIdx.x % nt;
   const int y = blockIdx.x * per + g;
@@ -162,7 +169,7 @@ __global__ void __launch_bounds__(kPupilThreads) k_pupil_out(const double2* plan
   __syncthreads();
   const double2* r = fft64_staged(b, b + M, M, 1, +1, tw, g < per ? t : M, nt);
   if (has) {
-    float2* d = out[blockIdx.y] + (size_t)y * mx;
+    float2* d = v.out[blockIdx.y] + (size_t)y * mx;
     for (int i = t; i < mx; i += nt) d[i] = make_float2((float)r[i].x, (float)r[i].y);
   }
 }
@@ -185,8 +192,8 @@ static bool fft64_length_ok(int L) {
 
 size_t pupil_scratch_bytes(const ls_plan* P, int n) { return (size_t)n * 2 * P->mx * P->my * sizeof(double2); }
 
-int apply_pupil_views(ls_plan* P, int n, const float2* const* in, float2* const* out, int adjoint, void* scratch,
-                      cudaStream_t st) {
+int apply_pupil_views(ls_plan* P, int n, const void* const* in, void* const* out, int adjoint, void* scratch,
+                      int scratch_views, cudaStream_t st) {
   const int mx = P->mx, my = P->my, Mx = 2 * mx, My = 2 * my;
   double2* d = static_cast<double2*>(scratch);
   const double2 *twx = twiddle64(Mx, st), *twy = twiddle64(My, st);
@@ -195,10 +202,19 @@ int apply_pupil_views(ls_plan* P, int n, const float2* const* in, float2* const*
   auto per = [](int L) { return std::max(1, std::min(8, 49152 / (int)(2 * L * sizeof(double2)))); };
   const int px = per(Mx), py = per(My);
   const size_t sx = (size_t)px * 2 * Mx * sizeof(double2), sy = (size_t)py * 2 * My * sizeof(double2);
-  k_pupil_rows<<<dim3((my + px - 1) / px, n), kPupilThreads, sx, st>>>(in, mx, my, px, d, twx);
-  k_pupil_cols<<<dim3((Mx + py - 1) / py, n), kPupilThreads, sy, st>>>(d, mx, my, py, P->pupil_h, adjoint,
-                                                                     1.0 / ((double)Mx * My), twy);
-  k_pupil_out<<<dim3((my + px - 1) / px, n), kPupilThreads, sx, st>>>(d, mx, my, px, out, twx);
+  const int most = std::min(scratch_views, PupilViews::kMax);
+  PupilViews v;
+  for (int q = 0; q < n; q += most) {
+    const int m = std::min(most, n - q);
+    for (int k = 0; k < m; ++k) {
+      v.in[k] = static_cast<const float2*>(in[q + k]);
+      v.out[k] = static_cast<float2*>(out[q + k]);
+    }
+    k_pupil_rows<<<dim3((my + px - 1) / px, m), kPupilThreads, sx, st>>>(v, mx, my, px, d, twx);
+    k_pupil_cols<<<dim3((Mx + py - 1) / py, m), kPupilThreads, sy, st>>>(d, mx, my, py, P->pupil_h, adjoint,
+                                                                       1.0 / ((double)Mx * My), twy);
+    k_pupil_out<<<dim3((my + px - 1) / px, m), kPupilThreads, sx, st>>>(d, mx, my, px, v, twx);
+  }
   LS_CUDA_TRY(cudaGetLastError());
   return LS_OK;
 }
@@ -264,23 +280,10 @@ int ls_apply_pupil(ls_plan* P, int n_views, const ls_c64* const* in, ls_c64* con
   cudaStream_t st = (cudaStream_t)stream;
   for (int q = 0; q < n_views; ++q)
     if (!in[q] || !out[q]) { set_last_error("null view pointer %d", q); return LS_EINVAL; }
-  // scratch planes and the two pointer tables in one stream-ordered allocation
-  const size_t planes = pupil_scratch_bytes(P, n_views);
-  char* scratch = nullptr;
-  LS_CUDA_TRY(cudaMallocAsync((void**)&scratch, planes + (size_t)2 * n_views * sizeof(void*), st));
-  void** tab = reinterpret_cast<void**>(scratch + planes);
-  std::vector<const void*> h(2 * (size_t)n_views);
-  for (int q = 0; q < n_views; ++q) {
-    h[q] = in[q];
-    h[n_views + q] = out[q];
-  }
-  int rc = LS_OK;
-  if (cudaMemcpyAsync(tab, h.data(), h.size() * sizeof(void*), cudaMemcpyHostToDevice, st) != cudaSuccess) {
-    set_last_error("pupil pointer table upload failed");
-    rc = LS_ECUDA;
-  }
-  if (rc == LS_OK)
-    rc = apply_pupil_views(P, n_views, (const float2* const*)tab, (float2* const*)(tab + n_views), adjoint, scratch, st);
+  const int most = std::min(n_views, PupilViews::kMax);
+  void* scratch = nullptr;
+  LS_CUDA_TRY(cudaMallocAsync(&scratch, pupil_scratch_bytes(P, most), st));
+  const int rc = apply_pupil_views(P, n_views, (const void* const*)in, (void* const*)out, adjoint, scratch, most, st);
   LS_CUDA_TRY(cudaFreeAsync(scratch, st));
   return rc;
 }

@@ -5,7 +5,7 @@ import pytest
 
 import phantoms as ph
 
-from gpu_common import H, KB, potential, to_dev, torch_and_lib
+from gpu_common import H, KB, LAM, potential, to_dev, torch_and_lib
 
 SHAPE = (16, 24, 32)
 
@@ -46,5 +46,27 @@ def test_replayed_batched_operator(views, how):
     torch.cuda.synchronize()
     for q in range(views):
         assert torch.equal(y[q], want[q]), q
+    del keep
+    plan.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("views", [3, 70])
+def test_replayed_pupil(views):
+    torch, ls = torch_and_lib()
+    plan = ls.Plan((8, 24, 24), KB, H)
+    ls.ls_set_pupil(plan.handle, 2 * np.pi * 0.9 / LAM, -1.7)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    a, b = (torch.view_as_complex(torch.randn((views, 24, 24, 2), device="cuda", generator=g)) for _ in range(2))
+    want = torch.empty_like(a)
+    ls.ls_apply_pupil(plan.handle, b, want)
+    x, y = a.clone(), torch.empty_like(a)
+    graph = _capture(torch, lambda: ls.ls_apply_pupil(plan.handle, x, y))
+    ls.ls_apply_pupil(plan.handle, a, torch.empty_like(a), True)
+    keep = _use_host_memory()
+    x.copy_(b)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
     del keep
     plan.close()
