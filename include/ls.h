@@ -369,7 +369,8 @@ enum ls_inject_kind {
   LS_INJECT_MAX_ROUNDS = 2,   /* plan: a solve's host loop stops after `value` rounds of launches; views    */
                               /*   still running report LS_TIMEOUT; value < 0 restores the normal bound     */
   LS_INJECT_ALLOC_FAIL = 3,   /* process-wide (plan may be NULL): the next `value` solver-workspace         */
-                              /*   allocations (plans and server lanes) fail with LS_ENOMEM                  */
+                              /*   allocations (plans and server lanes) fail with LS_ENOMEM; so do those of  */
+                              /*   ls_apply_pupil's scratch, which tries again with fewer views              */
   LS_INJECT_Z_STALL = 4,      /* plan: value > 0: the TMA-staged z pass waits on a barrier that nothing     */
                               /*   completes and gives up after `value` ns (every copy it issued is still    */
                               /*   waited for, with the normal one-second bound); the solve returns          */

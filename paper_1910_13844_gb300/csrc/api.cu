@@ -249,10 +249,10 @@ static int max_parts(const ls_plan* P) {
   return std::max(ix_blocks, 512);
 }
 
-// Test-only failure injection: the next g_fail_allocs engine allocations fail (ls_debug_inject).
+// Test-only failure injection: the next g_fail_allocs engine and pupil scratch allocations fail (ls_debug_inject).
 static std::atomic<long long> g_fail_allocs{0};
 
-static bool injected_alloc_failure() {
+bool injected_alloc_failure() {
   long long n = g_fail_allocs.load();
   while (n > 0)
     if (g_fail_allocs.compare_exchange_weak(n, n - 1)) return true;

@@ -148,6 +148,8 @@ int tune_forward(ls_plan* P, const float* f, int n, cudaStream_t st);
 // scratch holds pupil_scratch_bytes(P, scratch_views), scratch_views >= 1
 int apply_pupil_views(ls_plan* P, int n, const void* const* in, void* const* out, int adjoint, void* scratch,
                       int scratch_views, cudaStream_t st);
+// true: the allocation about to be made is to fail (ls_debug_inject)
+bool injected_alloc_failure();
 size_t pupil_scratch_bytes(const ls_plan* P, int n);
 
 // ls_matvec_noalloc set-up (noalloc.cu): the device address of the static scratch array on the

@@ -280,9 +280,16 @@ int ls_apply_pupil(ls_plan* P, int n_views, const ls_c64* const* in, ls_c64* con
   cudaStream_t st = (cudaStream_t)stream;
   for (int q = 0; q < n_views; ++q)
     if (!in[q] || !out[q]) { set_last_error("null view pointer %d", q); return LS_EINVAL; }
-  const int most = std::min(n_views, PupilViews::kMax);
+  // planes for all the views of a launch, or for as many as there is memory for
+  int most = std::min(n_views, PupilViews::kMax);
   void* scratch = nullptr;
-  LS_CUDA_TRY(cudaMallocAsync(&scratch, pupil_scratch_bytes(P, most), st));
+  for (;; most = (most + 1) / 2) {
+    const cudaError_t e = injected_alloc_failure() ? cudaErrorMemoryAllocation
+                                                   : cudaMallocAsync(&scratch, pupil_scratch_bytes(P, most), st);
+    if (e == cudaSuccess) break;
+    if (e != cudaErrorMemoryAllocation || most == 1) LS_CUDA_TRY(e);
+    cudaGetLastError();
+  }
   const int rc = apply_pupil_views(P, n_views, (const void* const*)in, (void* const*)out, adjoint, scratch, most, st);
   LS_CUDA_TRY(cudaFreeAsync(scratch, st));
   return rc;
