@@ -908,27 +908,6 @@ static int pupil_adjoint_residuals(ls_plan* P, int n, const ls_c64* const* r, cu
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// Caller memory that a batched call reads or writes while it runs.
-struct Spans {
-  struct Span { uintptr_t a, b; bool w; };
-  std::vector<Span> v;
-  void add(const void* p, size_t bytes, bool written) {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-    v.push_back({a, a + bytes, written});
-  }
-  // no written range overlaps another range
-  bool disjoint() {
-    std::sort(v.begin(), v.end(), [](const Span& x, const Span& y) { return x.a < y.a; });
-    uintptr_t any = 0, written = 0;
-    for (const Span& s : v) {
-      if (s.a < (s.w ? any : written)) return false;
-      any = std::max(any, s.b);
-      if (s.w) written = std::max(written, s.b);
-    }
-    return true;
-  }
-};
-
 static int worst_status(const Engine& e, int nslots, ls_stats* stats) {
   int worst = LS_OK;
   for (int s = 0; s < nslots; ++s) {

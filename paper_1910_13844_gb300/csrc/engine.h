@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "common.cuh"
@@ -151,6 +152,27 @@ int apply_pupil_views(ls_plan* P, int n, const void* const* in, void* const* out
 // true: the allocation about to be made is to fail (ls_debug_inject)
 bool injected_alloc_failure();
 size_t pupil_scratch_bytes(const ls_plan* P, int n);
+
+// Caller memory that a batched call reads or writes while it runs.
+struct Spans {
+  struct Span { uintptr_t a, b; bool w; };
+  std::vector<Span> v;
+  void add(const void* p, size_t bytes, bool written) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    v.push_back({a, a + bytes, written});
+  }
+  // no written range overlaps another range
+  bool disjoint() {
+    std::sort(v.begin(), v.end(), [](const Span& x, const Span& y) { return x.a < y.a; });
+    uintptr_t any = 0, written = 0;
+    for (const Span& s : v) {
+      if (s.a < (s.w ? any : written)) return false;
+      any = std::max(any, s.b);
+      if (s.w) written = std::max(written, s.b);
+    }
+    return true;
+  }
+};
 
 // ls_matvec_noalloc set-up (noalloc.cu): the device address of the static scratch array on the
 // current device; loads the array's module (reserving the array) if that has not happened yet.

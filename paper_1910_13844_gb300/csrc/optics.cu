@@ -202,7 +202,14 @@ int apply_pupil_views(ls_plan* P, int n, const void* const* in, void* const* out
   auto per = [](int L) { return std::max(1, std::min(8, 49152 / (int)(2 * L * sizeof(double2)))); };
   const int px = per(Mx), py = per(My);
   const size_t sx = (size_t)px * 2 * Mx * sizeof(double2), sy = (size_t)py * 2 * My * sizeof(double2);
-  const int most = std::min(scratch_views, PupilViews::kMax);
+  // a view whose output is another's input or output waits for it, as it did one view at a time
+  Spans io;
+  for (int q = 0; q < n; ++q) {
+    const size_t bytes = (size_t)mx * my * sizeof(float2);
+    io.add(out[q], bytes, true);
+    if (in[q] != out[q]) io.add(in[q], bytes, false);
+  }
+  const int most = io.disjoint() ? std::min(scratch_views, PupilViews::kMax) : 1;
   PupilViews v;
   for (int q = 0; q < n; q += most) {
     const int m = std::min(most, n - q);

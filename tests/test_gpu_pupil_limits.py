@@ -1,4 +1,4 @@
-"""ls_apply_pupil where it cannot take all views at once: no memory for their scratch."""
+"""ls_apply_pupil where it cannot take all views at once: no memory for their scratch, or views that share memory."""
 import numpy as np
 import pytest
 
@@ -42,4 +42,32 @@ def test_no_scratch_at_all():
     assert err.value.code == ls.LS_ENOMEM
     ls.ls_apply_pupil(plan.handle, y, y)
     torch.cuda.synchronize()
+    plan.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("how", ["chain", "one output", "shifted", "both in place"])
+def test_views_that_share_memory_run_in_order(how):
+    torch, ls = torch_and_lib()
+    m = 24
+
+    def vectors():
+        pool = torch.view_as_complex(torch.randn((5 * m * m, 2), device="cuda", generator=torch.Generator("cuda").manual_seed(3)))
+        v = [pool[q * m * m:(q + 1) * m * m] for q in range(5)]
+        if how == "chain":
+            return pool, v[:4], v[1:]
+        if how == "one output":
+            return pool, v[:3], [v[4]] * 3
+        if how == "shifted":
+            return pool, v[1:4], [pool[q * m * m + m:(q + 1) * m * m + m] for q in range(3)]
+        return pool, [v[0], v[0]], [v[0], v[0]]
+
+    plan, _ = _plan(torch, ls, 1)
+    want, x, y = vectors()
+    for a, b in zip(x, y):
+        ls.ls_apply_pupil(plan.handle, [a], [b])
+    got, x, y = vectors()
+    ls.ls_apply_pupil(plan.handle, x, y)
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)
     plan.close()
