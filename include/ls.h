@@ -64,7 +64,11 @@ enum ls_status {
 };
 
 typedef struct { int nx, ny, nz; } ls_grid;      /* voxels per axis, each in {8,12,16,24,32,48,64,72,96,128,144,192} */
-typedef struct { float re, im; } ls_c64;
+typedef struct { float re, im; } ls_c64;   /* vectors: see "alignment" below */
+
+/* Alignment: vectors of ls_c64 should lie on 16 bytes and have to lie on 8, but for those that
+ * ls_matvec_batch, ls_forward, ls_forward_warm and ls_farfield read or write, the u_in of
+ * ls_gradient and the out of ls_farfield_adjoint: these may lie on 4 and are copied. */
 
 typedef struct {
   double tol;          /* BiCGStab stop: ||r|| <= tol ||b|| (recursive residual).  Default 1e-6.      */

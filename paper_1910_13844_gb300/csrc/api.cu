@@ -884,14 +884,14 @@ void prof_resolve(ls_plan* P, bool wait) {
   pr.pending.resize(keep);
 }
 
-// far[q] <- P e.far[q] for slots [0, n) (no-op without a pupil).  The A1 buffers (16 nz bytes for each of the
+// out[q] <- P e.far[q] for slots [0, n) (out null: in place; no-op without a pupil).  The A1 buffers (16 nz bytes for each of the
 // 2 nx ny columns of a slot's plane) are free once the far field is done and hold the scratch planes.
-static int pupil_on_far(ls_plan* P, int n, ls_c64* const* far, cudaStream_t st) {
+static int pupil_on_far(ls_plan* P, int n, ls_c64* const* out, cudaStream_t st) {
   if (!P->pupil_h) return LS_OK;
   Engine& e = P->eng;
-  std::vector<const void*> src(n);
+  std::vector<void*> src(n);
   for (int q = 0; q < n; ++q) src[q] = e.far + (size_t)q * P->mx * P->my;
-  return apply_pupil_views(P, n, src.data(), (void* const*)far, 0, e.a1, n, st);
+  return apply_pupil_views(P, n, src.data(), out ? (void* const*)out : src.data(), 0, e.a1, n, st);
 }
 
 // Uploads the table (1) of the residuals that G~^H is applied to: r_q, or P^H r_q in the engine's detector
@@ -906,6 +906,13 @@ static int pupil_adjoint_residuals(ls_plan* P, int n, const ls_c64* const* r, cu
   return apply_pupil_views(P, n, (const void* const*)r, dst.data(), 1, e.a1, n, st);
 }
 
+// ls_c64 is two floats: a vector need not lie on 8 bytes, but the kernels' complex loads and stores do.
+static bool aligned8(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7) == 0; }
+static bool aligned8(const ls_c64* const* v, int n) {
+  for (int q = 0; v && q < n; ++q)
+    if (!aligned8(v[q])) return false;
+  return true;
+}
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 static int worst_status(const Engine& e, int nslots, ls_stats* stats) {
@@ -1250,13 +1257,14 @@ int ls_matvec_batch(ls_plan* P, const float* f, int n_views, const ls_c64* const
   if (rc) return rc;
   Engine& e = P->eng;
   // The passes read x[q] and write y[q] where they are; in place (y[q] == x[q]) each element is read by
-  // the thread that writes it.  Where an output overlaps another vector the call works on copies.
+  // the thread that writes it.  Where an output overlaps another vector, or one does not lie on 8 bytes, the
+  // call works on copies.
   Spans io;
   for (int q = 0; q < n_views; ++q) {
     io.add(y[q], e.N * sizeof(float2), true);
     if (x[q] != y[q]) io.add(x[q], e.N * sizeof(float2), false);
   }
-  const bool direct = io.disjoint();
+  const bool direct = io.disjoint() && aligned8(x, n_views) && aligned8(y, n_views);
   // the call does not synchronise and may be captured: the slot states go out as kernel arguments
   OperatorSlots s;
   s.f = f;
@@ -1322,8 +1330,8 @@ static int builtin_plane_waves(ls_plan* P, int n, cudaStream_t st) {
 // initial guesses x0 (NULL: the right-hand sides).  The solve reads the caller's right-hand sides and
 // guesses where they are and updates the fields in out[q] (NULL: in the workspace), unless `copy` (an
 // output overlaps another of the call's vectors): then it works on copies in the workspace.  Fields are
-// read and written 16 bytes at a time by the update, so a pointer that is not so aligned takes the
-// workspace too.
+// read and written 16 bytes at a time by the update, right-hand sides 8 bytes at a time, so a pointer that is
+// not so aligned takes the workspace too.
 static int load_rhs(ls_plan* P, const float* f, int n, const ls_c64* const* rhs, const ls_c64* const* x0, bool copy,
                     float2* const* out, cudaStream_t st) {
   Engine& e = P->eng;
@@ -1334,7 +1342,7 @@ static int load_rhs(ls_plan* P, const float* f, int n, const ls_c64* const* rhs,
   for (int q = 0; q < n; ++q) {
     SlotDev& s = e.slots_h[q];
     slot_defaults(P, s, q, f, 0);
-    if (rhs && copy)
+    if (rhs && (copy || !aligned8(rhs[q])))
       LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_B, q), rhs[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
     else if (rhs)
       s.b = (const float2*)rhs[q];
@@ -1380,17 +1388,17 @@ static int forward_impl(ls_plan* P, const float* f, int n_views, const ls_c64* c
   const bool copy = !io.disjoint();
   rc = load_rhs(P, f, n_views, u_in, x0, copy, (float2* const*)u_out, st);
   if (rc) return rc;
-  const bool far_direct = far && !copy && !P->pupil_h;
-  if (far_direct)
+  const bool far_direct = far && !copy && aligned8(far, n_views);
+  if (far_direct && !P->pupil_h)
     for (int q = 0; q < n_views; ++q) e.slots_h[q].far = (float2*)far[q];
   rc = engine_solve(P, n_views, st);
   if (rc) return rc;
   const int status = worst_status(e, n_views, stats);
   if (far) {
     seq_far(P, n_views, 0, st);
-    rc = pupil_on_far(P, n_views, far, st);
+    rc = pupil_on_far(P, n_views, far_direct ? far : nullptr, st);
     if (rc) return rc;
-    if (!far_direct && !P->pupil_h)
+    if (!far_direct)
       for (int q = 0; q < n_views; ++q)
         LS_CUDA_TRY(cudaMemcpyAsync(far[q], e.far + (size_t)q * P->mx * P->my, db, cudaMemcpyDeviceToDevice, st));
   }
@@ -1424,17 +1432,25 @@ int ls_farfield(ls_plan* P, const float* f, int n_views, const ls_c64* const* u,
   rc = engine_reserve(P, n_views);
   if (rc) return rc;
   Engine& e = P->eng;
-  // the fields are read, and (without a pupil) the far fields written, where they are: every field has
+  // the fields are read and the far fields written where they are (if they lie on 8 bytes): every field has
   // been read before the first far field is written
+  const size_t db = (size_t)P->mx * P->my * sizeof(float2);
+  const bool direct = aligned8(far, n_views);
   for (int q = 0; q < n_views; ++q) {
     slot_defaults(P, e.slots_h[q], q, f, 0);
-    e.slots_h[q].x = (const float2*)u[q];
-    if (!P->pupil_h) e.slots_h[q].far = (float2*)far[q];
+    if (aligned8(u[q]))
+      e.slots_h[q].x = (const float2*)u[q];
+    else
+      LS_CUDA_TRY(cudaMemcpyAsync(e.vptr(V_X, q), u[q], e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+    if (direct && !P->pupil_h) e.slots_h[q].far = (float2*)far[q];
   }
   LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, e.slots_h, (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
   seq_far(P, n_views, 0, st);
-  rc = pupil_on_far(P, n_views, far, st);
+  rc = pupil_on_far(P, n_views, direct ? far : nullptr, st);
   if (rc) return rc;
+  if (!direct)
+    for (int q = 0; q < n_views; ++q)
+      LS_CUDA_TRY(cudaMemcpyAsync(far[q], e.far + (size_t)q * P->mx * P->my, db, cudaMemcpyDeviceToDevice, st));
   LS_CUDA_TRY(cudaStreamSynchronize(st));
   return LS_OK;
 }
@@ -1451,13 +1467,17 @@ int ls_farfield_adjoint(ls_plan* P, int n_views, const ls_c64* const* r, ls_c64*
   Engine& e = P->eng;
   rc = pupil_adjoint_residuals(P, n_views, r, st);
   if (rc) return rc;
-  // the outputs are written last, where they are: every residual has been read by then
+  // the outputs are written last, where they are (if they lie on 8 bytes): every residual has been read by then
+  const bool direct = aligned8(out, n_views);
   for (int q = 0; q < n_views; ++q) {
     slot_defaults(P, e.slots_h[q], q, nullptr, 1);
-    e.slots_h[q].bo = (float2*)out[q];
+    if (direct) e.slots_h[q].bo = (float2*)out[q];
   }
   LS_CUDA_TRY(cudaMemcpyAsync(e.slots_d, e.slots_h, (size_t)n_views * sizeof(SlotDev), cudaMemcpyHostToDevice, st));
   seq_far_adjoint(P, n_views, (const float2* const*)engine_ptr_table(P, 1), 0, st);
+  if (!direct)
+    for (int q = 0; q < n_views; ++q)
+      LS_CUDA_TRY(cudaMemcpyAsync(out[q], e.vptr(V_B, q), e.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
   LS_CUDA_TRY(cudaStreamSynchronize(st));
   return LS_OK;
 }
