@@ -1234,6 +1234,14 @@ int ls_matvec(ls_plan* P, const float* f, const ls_c64* x, ls_c64* y, int adjoin
   return single_op(P, f, x, y, adjoint, 1, (cudaStream_t)stream);
 }
 
+// The passes may write these outputs where they are: on 8 bytes, and no two overlapping (overlapping ones are
+// copied out in the order of the views).
+static bool separate_outputs(const ls_c64* const* out, int n, size_t bytes) {
+  Spans io;
+  for (int q = 0; q < n; ++q) io.add(out[q], bytes, true);
+  return aligned8(out, n) && io.disjoint();
+}
+
 static int check_views(int n, const void* const* a, const char* what, bool allow_null_array) {
   if (!a) {
     if (allow_null_array) return LS_OK;
@@ -1432,10 +1440,10 @@ int ls_farfield(ls_plan* P, const float* f, int n_views, const ls_c64* const* u,
   rc = engine_reserve(P, n_views);
   if (rc) return rc;
   Engine& e = P->eng;
-  // the fields are read and the far fields written where they are (if they lie on 8 bytes): every field has
-  // been read before the first far field is written
+  // the fields are read and the far fields written where they are: every field has been read before the first
+  // far field is written
   const size_t db = (size_t)P->mx * P->my * sizeof(float2);
-  const bool direct = aligned8(far, n_views);
+  const bool direct = separate_outputs(far, n_views, db);
   for (int q = 0; q < n_views; ++q) {
     slot_defaults(P, e.slots_h[q], q, f, 0);
     if (aligned8(u[q]))
@@ -1467,8 +1475,8 @@ int ls_farfield_adjoint(ls_plan* P, int n_views, const ls_c64* const* r, ls_c64*
   Engine& e = P->eng;
   rc = pupil_adjoint_residuals(P, n_views, r, st);
   if (rc) return rc;
-  // the outputs are written last, where they are (if they lie on 8 bytes): every residual has been read by then
-  const bool direct = aligned8(out, n_views);
+  // the outputs are written last, where they are: every residual has been read by then
+  const bool direct = separate_outputs(out, n_views, e.N * sizeof(float2));
   for (int q = 0; q < n_views; ++q) {
     slot_defaults(P, e.slots_h[q], q, nullptr, 1);
     if (direct) e.slots_h[q].bo = (float2*)out[q];
