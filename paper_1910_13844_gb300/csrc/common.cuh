@@ -106,6 +106,9 @@ struct SlotDev {
 // grids they let their CTAs be placed while the kernel before them drains (launch_pdl), and wait for that
 // kernel's completion before they touch memory (pdl_begin, the first statement of every CTA: a kernel
 // completes only after the one before it has).  Launched without the attribute the wait returns at once.
+// So what an earlier kernel of the solver wrote is not read-only for the lifetime of the next one, which may begin
+// before: such vectors are read with plain loads, never __ldg (ld.global.nc), which is kept for tables, spectra and
+// the potential.  The same goes for a vector that the kernel itself may write (the operator in place).
 // Small: below 2^20 voxels.  Measured without and with: forward at 32^3 x 1 292 -> 274 us, a served burst
 // at 64^3 12.5 -> 11.9 ms, gradient at 96^3 x 16 7.68 -> 7.62 ms; but 144^3 x 1 5.38 -> 5.41 ms, the operator
 // at 128^3 x 60 4.37 -> 4.52 ms.

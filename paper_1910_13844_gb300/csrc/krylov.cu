@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(256, 4) k_update(UpdParams a) {
   const size_t n4 = a.n / 2;
   float acc[3] = {0.f, 0.f, 0.f};
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    float4 pv = __ldg(p + i), sv = __ldg(s + i), tv = __ldg(t + i), hv = __ldg(rh + i), xv = xi[i];
+    float4 pv = p[i], sv = s[i], tv = t[i], hv = rh[i], xv = xi[i];
     float2 p0 = make_float2(pv.x, pv.y), p1 = make_float2(pv.z, pv.w);
     float2 s0 = make_float2(sv.x, sv.y), s1 = make_float2(sv.z, sv.w);
     float2 t0 = make_float2(tv.x, tv.y), t1 = make_float2(tv.z, tv.w);
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(256) k_far_reduce(FarPassParams a) {
   const float2* k = a.k2 + i;
   float2 acc = make_float2(0.f, 0.f);
 #pragma unroll 8
-  for (int z = z0; z < z1; ++z) acc = cadd(acc, cmul(__ldg(k + (size_t)z * plane), __ldg(src + (size_t)z * plane)));
+  for (int z = z0; z < z1; ++z) acc = cadd(acc, cmul(__ldg(k + (size_t)z * plane), src[(size_t)z * plane]));
   a.dst[(size_t)slot * a.dst_stride + blockIdx.z * plane + i] = acc;
 }
 

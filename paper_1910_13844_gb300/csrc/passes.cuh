@@ -137,26 +137,27 @@ __device__ __forceinline__ void fx_body(const FxParams& a) {
       if (!LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)row * nx + x, (size_t)a.rows * nx, a.vstride),
                         BS_FX_VEC))
         continue;
-      float2 val = __ldg(src + x);
-      if (a.mode == FX_BICG_P) {
-        if (!first) {
-          // p = r + beta (p - omega v)
-          float2 pv = a.vp[i], vv = __ldg(a.vv + i);
-          float2 d = csub(pv, cmul(make_float2(om_re, om_im), vv));
-          val = cadd(val, cmul(make_float2(fa, fb), d));
-        }
-        a.vp[i] = val;
+      float2 val = src[x];
+      if (a.mode == FX_BICG_P && !first) {
+        // p = r + beta (p - omega v)
+        float2 d = csub(a.vp[i], cmul(make_float2(om_re, om_im), a.vv[i]));
+        val = cadd(val, cmul(make_float2(fa, fb), d));
       } else if (a.mode == FX_BICG_S) {
         // s = r - alpha v
-        float2 vv = __ldg(a.vv + i);
-        val = csub(val, cmul(make_float2(al_re, al_im), vv));
-        a.vs[i] = val;
-      }
-      if (a.mode != FX_COPY) {
-        const float fv = __ldg(f + (size_t)row * nx + x);
-        val = cscale(val, fv);
+        val = csub(val, cmul(make_float2(al_re, al_im), a.vv[i]));
       }
       v[n1] = val;
+    }
+    // the stores after all the loads, which the compiler cannot move across them
+#pragma unroll
+    for (int n1 = 0; n1 < R1 / 2; ++n1) {
+      const int x = R2 * n1 + t;
+      if (!LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)row * nx + x, (size_t)a.rows * nx, a.vstride),
+                        BS_FX_VEC))
+        continue;
+      if (a.mode == FX_BICG_P) a.vp[voff + x] = v[n1];
+      else if (a.mode == FX_BICG_S) a.vs[voff + x] = v[n1];
+      if (a.mode != FX_COPY) v[n1] = cscale(v[n1], __ldg(f + (size_t)row * nx + x));
     }
   }
   float2* S = sm + (size_t)p * G::XROW;
@@ -386,7 +387,7 @@ __device__ __forceinline__ void strided_body(const StridedParams& a) {
       if ((DIR < 0 ? (n1 < R1 / 2) : true) &&
           LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)plane * a.src_plane + (size_t)y * a.ncont + c,
                                     src_ext, a.src_stride), BS_ST_SRC))
-        v[n1] = __ldg(src + (size_t)y * a.ncont);
+        v[n1] = src[(size_t)y * a.ncont];
     }
   }
   if (t < R2) {
@@ -465,13 +466,13 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PS) k_far_iy(FarPassParams
 #pragma unroll
         for (int n1 = 0; n1 < R1; ++n1) {
           const size_t o = (size_t)(R2 * n1 + t) * a.ncont;
-          v[n1] = cmulc(__ldg(src + o), __ldg(k + o));
+          v[n1] = cmulc(src[o], __ldg(k + o));
         }
       } else {
         for (int q = 0; q < a.zchunks; ++q) {
 #pragma unroll
           for (int n1 = 0; n1 < R1; ++n1)
-            v[n1] = cadd(v[n1], __ldg(src + q * plane + (size_t)(R2 * n1 + t) * a.ncont));
+            v[n1] = cadd(v[n1], src[q * plane + (size_t)(R2 * n1 + t) * a.ncont]);
         }
       }
     }
@@ -539,7 +540,7 @@ __device__ __forceinline__ void ix_body(const IxParams& a) {
       const size_t o = TR ? (size_t)(R2 * n1 + t1) * a.rows : (size_t)(R2 * n1 + t1);
       if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, o + (TR ? (size_t)row1 : (size_t)row1 * L), (size_t)a.rows * L,
                                     a.src_stride), BS_IX_SRC))
-        v[n1] = __ldg(s + o);
+        v[n1] = s[o];
     }
   }
   if (t1 < R2) {
@@ -561,50 +562,69 @@ __device__ __forceinline__ void ix_body(const IxParams& a) {
     float2* out0 = a.out0 ? a.out0 + sbase
                    : a.out_slot == IX_OUT_XO ? a.sel.slots[slot].xo
                    : a.out_slot == IX_OUT_FAR ? a.sel.slots[slot].far : a.sel.slots[slot].bo;
+    // g = u[k2] becomes the result, then the results are stored: the loads come before all the stores, which the
+    // compiler cannot move them across (in0 may be out0)
+    auto elem = [&](int k2) { return (size_t)row * nx + t + R1 * k2; };
+    auto ok = [&](int k2) {
+      return LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, elem(k2), (size_t)a.rows * nx, a.vstride), BS_IX_VEC);
+    };
+    switch (a.mode) {
+      case IX_STORE:
 #pragma unroll
-    for (int k2 = 0; k2 < R2 / 2; ++k2) {
-      const int x = t + R1 * k2;
-      const float2 g = u[k2];
-      const size_t i = (size_t)row * nx + x;
-      if (!LS_IN_BOUNDS(a.mode == IX_STORE ||
-                            slot_elem_ok(slot, a.sel.nslots, (size_t)row * nx + x, (size_t)a.rows * nx, a.vstride),
-                        BS_IX_VEC))
-        continue;
-      switch (a.mode) {
-        case IX_STORE: {
-          const int xo = x - a.out_o;
+        for (int k2 = 0; k2 < R2 / 2; ++k2) {
+          const int xo = t + R1 * k2 - a.out_o;
           if (xo >= 0 && xo < a.out_m &&
               LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, (size_t)row * a.out_m + xo, (size_t)a.rows * a.out_m,
                                         a.vstride), BS_IX_VEC))
-            out0[(size_t)row * a.out_m + xo] = g;
-        } break;
-        case IX_MATVEC:
-          out0[i] = csub(__ldg(in0 + i), g);
-          break;
-        case IX_BICG_V: {
-          float2 vv = csub(__ldg(in0 + i), g);
-          out0[i] = vv;
-          float2 d = cdotterm(__ldg(in1 + i), vv);   // conj(rh) v
-          acc[0] += d.x; acc[1] += d.y;
-          acc[2] += vv.x * vv.x + vv.y * vv.y;          // ||v||^2 (relative breakdown test)
-        } break;
-        case IX_BICG_T: {
-          float2 ss = __ldg(in0 + i);
-          float2 tt = csub(ss, g);
-          out0[i] = tt;
-          float2 d = cdotterm(tt, ss);                  // conj(t) s
-          acc[0] += d.x; acc[1] += d.y;
-          acc[2] += tt.x * tt.x + tt.y * tt.y;
-        } break;
-        case IX_RESID: {
-          float2 b = __ldg(in1 + i);
-          float2 r = cadd(csub(b, __ldg(in0 + i)), g);   // b - (x - G f x)
-          out0[i] = r;
-          a.out1[sbase + i] = r;
-          acc[0] += r.x * r.x + r.y * r.y;
-          acc[1] += b.x * b.x + b.y * b.y;
-        } break;
-      }
+            out0[(size_t)row * a.out_m + xo] = u[k2];
+        }
+        break;
+      case IX_MATVEC:
+#pragma unroll
+        for (int k2 = 0; k2 < R2 / 2; ++k2)
+          if (ok(k2)) u[k2] = csub(in0[elem(k2)], u[k2]);
+        break;
+      case IX_BICG_V:
+#pragma unroll
+        for (int k2 = 0; k2 < R2 / 2; ++k2)
+          if (ok(k2)) {
+            const float2 vv = csub(in0[elem(k2)], u[k2]);
+            u[k2] = vv;
+            const float2 d = cdotterm(in1[elem(k2)], vv);   // conj(rh) v
+            acc[0] += d.x; acc[1] += d.y;
+            acc[2] += vv.x * vv.x + vv.y * vv.y;            // ||v||^2 (relative breakdown test)
+          }
+        break;
+      case IX_BICG_T:
+#pragma unroll
+        for (int k2 = 0; k2 < R2 / 2; ++k2)
+          if (ok(k2)) {
+            const float2 ss = in0[elem(k2)], tt = csub(ss, u[k2]);
+            u[k2] = tt;
+            const float2 d = cdotterm(tt, ss);              // conj(t) s
+            acc[0] += d.x; acc[1] += d.y;
+            acc[2] += tt.x * tt.x + tt.y * tt.y;
+          }
+        break;
+      case IX_RESID:
+#pragma unroll
+        for (int k2 = 0; k2 < R2 / 2; ++k2)
+          if (ok(k2)) {
+            const float2 b = in1[elem(k2)];
+            const float2 r = cadd(csub(b, in0[elem(k2)]), u[k2]);   // b - (x - G f x)
+            u[k2] = r;
+            acc[0] += r.x * r.x + r.y * r.y;
+            acc[1] += b.x * b.x + b.y * b.y;
+          }
+        break;
+    }
+    if (a.mode != IX_STORE) {
+#pragma unroll
+      for (int k2 = 0; k2 < R2 / 2; ++k2)
+        if (ok(k2)) {
+          out0[elem(k2)] = u[k2];
+          if (a.mode == IX_RESID) a.out1[sbase + elem(k2)] = u[k2];
+        }
     }
   }
   if (a.mode >= IX_BICG_V && LS_IN_BOUNDS(a.maxparts == 0 || (int)gridDim.x <= a.maxparts, BS_IX_PART)) {
