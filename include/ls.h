@@ -248,9 +248,10 @@ int ls_prox_hs(const ls_grid* grid, const float* z, float* x, double lam, int it
  * plan's check_every / use_graphs options are overwritten).  If the environment variable
  * LS_AUTOTUNE_CACHE names a file, a result for the same device, grid and view count is read from it
  * instead of timing, and new results are appended to it (a line's last field says whether FY, Z and
- * IY run as one fused pass; lines without it run the three).  The z-pass form chosen, fused or not,
- * applies to launches of more than n_views / 2 views; smaller batches on the same plan keep the per-length default form
- * (the fastest form depends on the batch size).  Synchronous; uses the plan's workspace (its
+ * IY run as one fused pass; lines without it run the three).  The choice between the fused pass and
+ * the three applies to batches of more than n_views / 2 views, in all their launches; the z-pass form chosen to
+ * launches of more than n_views / 2 views.  Smaller ones on the same plan keep the per-length defaults (the
+ * fastest form depends on the batch size).  Synchronous; uses the plan's workspace (its
  * contents are overwritten).  out may be NULL.  No counterpart in the paper. */
 int ls_autotune(ls_plan* plan, int n_views, const float* f, ls_tune* out, void* cuda_stream);
 

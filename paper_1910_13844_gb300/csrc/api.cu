@@ -406,12 +406,13 @@ static SlotSel counted(ls_plan* P, SlotSel s, int kind) {
 }
 
 // Whether a launch over nslots views runs the fused y/z pass: where (ny, nz) has one, as ls_autotune chose
-// for launches of more than half the tuned batch, else by the pair's measured rule (YZ::large_ok: always,
-// or for launches of at most two waves of its CTAs, where the launches saved count most).  The z pass's
-// waits are under test only in the five-pass form.
+// for batches of more than half the tuned one (whatever the chunks they are launched in), else by the
+// pair's measured rule (YZ::large_ok: always, or for launches of at most two waves of its CTAs, where the
+// launches saved count most).  The z pass's waits are under test only in the five-pass form.
 static bool use_fused(const ls_plan* P, int nslots) {
   if (!P->gyz || P->inj_z_stall || P->inj_z_wait_ns) return false;
-  if (P->tune_fused >= 0 && 2 * nslots > P->tune_views) return P->tune_fused != 0;
+  const int batch = P->batch_views > 0 ? P->batch_views : nslots;
+  if (P->tune_fused >= 0 && 2 * batch > P->tune_views) return P->tune_fused != 0;
   return P->yz.large_ok || (long long)P->nx * nslots <= (long long)P->sms * P->yz.minb;
 }
 
@@ -577,6 +578,7 @@ void seq_iter_chunked(ls_plan* P, int nslots, cudaStream_t st) {
   }
   for (int s0 = 0; s0 < nslots; s0 += c) {
     ls_plan v = plan_slot_view(P, s0);
+    v.batch_views = nslots;
     seq_iter(&v, std::min(c, nslots - s0), st);
   }
 }

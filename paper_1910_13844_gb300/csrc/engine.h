@@ -96,8 +96,10 @@ struct ls_plan {
                                   // more than tune_views / 2 views, smaller launches take the ZAuto form
   int tune_fx_bulk = -1;          // bulk-copy-staged persistent first pass (-1, untuned: the length's FxBulk)
   int tune_strided_wide = 0;      // FY/IY with 32 pencils per CTA (else 16)
-  int tune_fused = -1;            // fused y/z pass: 1 on, 0 off, -1 (untuned) where it exists
+  int tune_fused = -1;            // fused y/z pass: 1 on, 0 off (batches of more than tune_views / 2 views, in all
+                                  // their launches), -1 (untuned) by use_fused's rule
   int tune_views_per_launch = 0;  // BiCGStab iteration launched over chunks of this many views (0: all)
+  int batch_views = 0;            // a slot view whose launches are chunks of a batch: the batch's views (else 0)
   // test-only failure injection (ls_debug_inject); the defaults inject nothing
   int inj_zero_shadow_view = -1;  // this view's shadow residual is zeroed at the start of a solve
   long long inj_max_rounds = -1;  // host rounds a solve may take (-1: the normal bound)
