@@ -8,12 +8,12 @@
 //   * FY / IY: 16 or 32 pencils per CTA;
 //   * IX: L2 prefetch of its epilogue operands at kernel start, or not;
 //   * FX: launch grid with the views fastest (shared potential rows from L2), or the rows fastest;
+//   * these two beside the fused y/z pass too, which then stands against FY, Z and IY in the solve loop;
 //   * the solve loop: FX in the BiCGStab iteration as the bulk-copy-staged persistent kernel (input rows
 //     staged in shared memory, three row blocks ahead) or not, the views per launch of an iteration
 //     (all, or chunks of n/2, n/4 or 8 views, each chunk one launch per pass), iterations between
 //     host reads of the convergence mask (2, 4, 8), and replay of the iteration from a captured CUDA
-//     graph or direct launches;
-//   * the fused y/z pass instead of FY, Z and IY, before the loop variants.
+//     graph or direct launches.
 // Operator variants are timed on batched operator applications, the loop variants on forward solves
 // of plane-wave illuminations.  Every operator variant's output is first compared with the default
 // variants' (relative L2 over the batch); a variant that differs by more than 1e-5 is never chosen.
@@ -242,16 +242,26 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
   if (e.a2_map_ok && P->zwa2_z) mv_ms = tune_op(&cur.z_split, 2, two);
   if (e.a2_map_ok) mv_ms = tune_op(&cur.z_tma, 2, two);
   mv_ms = tune_op(&cur.strided_wide, 2, two);
-  mv_ms = tune_op(&cur.ix_prefetch, 2, two);
-  mv_ms = tune_op(&cur.fx_views_fastest, 2, two);
-  // the fused y/z pass: its operator now (the reference output is still there), its solves below
-  double fused_ms = -1.0;
-  if (P->gyz) {
-    apply(P, cur, 1);
-    const double dev = deviation();
-    if (dev >= 0.0 && dev <= 1e-5) fused_ms = time_ms(st, 3, matvec);
-    apply(P, cur, 0);
+  // FX and IX have another layout on their far side with the fused y/z pass: their knobs for either form now
+  // (the reference output is still there), its solves below
+  struct { int ix_prefetch, fx_views_fastest; double ms; } form[2] = {{0, 0, -1.0}, {0, 0, -1.0}};
+  const int start_prefetch = cur.ix_prefetch, start_fastest = cur.fx_views_fastest;
+  for (fused = P->gyz ? 1 : 0; fused >= 0; --fused) {
+    cur.ix_prefetch = start_prefetch;
+    cur.fx_views_fastest = start_fastest;
+    tune_op(&cur.ix_prefetch, 2, two);
+    form[fused].ms = tune_op(&cur.fx_views_fastest, 2, two);   // negative: no variant gave the operator
+    form[fused].ix_prefetch = cur.ix_prefetch;
+    form[fused].fx_views_fastest = cur.fx_views_fastest;
   }
+  auto set_form = [&](int k) {
+    fused = k;
+    cur.ix_prefetch = form[k].ix_prefetch;
+    cur.fx_views_fastest = form[k].fx_views_fastest;
+    mv_ms = form[k].ms;
+    apply(P, cur, fused);
+  };
+  set_form(0);
   // solve loop: forward solves of the plane waves
   auto solve = [&] { return tune_forward(P, f, n_views, st); };
   auto solve_views = solve;
@@ -260,15 +270,11 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
     // the fused y/z pass in place of the three (tuned) passes, where the grid has it: before the launch
     // structure, whose best differs (60 views at 128^3: 30 a launch with three passes, whose intermediates are
     // larger, all 60 with one; the choice made for three passes cost a solve with one 3%)
-    if (fused_ms > 0) {
-      apply(P, cur, 0);
+    if (form[1].ms > 0) {
       const double three = time_ms(st, kSolveReps, solve);
-      apply(P, cur, 1);
+      set_form(1);
       const double one = time_ms(st, kSolveReps, solve);
-      if (one > 0 && (three < 0 || one < three)) {
-        fused = 1;
-        mv_ms = fused_ms;
-      }
+      if (!(one > 0 && (three < 0 || one < three))) set_form(0);
     }
     // the bulk-staged first pass in the iteration: its solution must equal the plain kernel's
     // (the same arithmetic in the same order) before its time counts; the reference solution is kept

@@ -69,3 +69,22 @@ def test_chunks_of_a_pair_that_is_fused_only_by_choice(tmp_path, monkeypatch):
     torch_and_lib()
     line = "1 1 0 2 0 1.0 1.0 0 0 40 0 0 1"
     assert set(solve_forms(tmp_path, monkeypatch, (8, 32, 64), 80, line)) == {True}
+
+
+@pytest.mark.gpu
+def test_the_tuner_tries_the_first_and_last_pass_in_both_forms(tmp_path):
+    # before its first solve: the prefetch and the grid order, two values each, in the three passes and the fused one
+    torch_and_lib()
+    lines = _run(tmp_path, """
+        import torch
+        import paper_1910_13844_gb300 as ls
+        plan = ls.Plan((16, 16, 16), 8.0, 0.1)
+        t = plan.autotune(2, torch.full((16, 16, 16), 0.5, device="cuda"))
+        assert t["from_cache"] == 0
+        plan.close()
+    """)
+    before = lines[:lines.index("push solve")]
+    runs = [b == "push Z" for a, b in zip(before, before[1:]) if a == "push FY"]
+    per_variant = 1 + 4   # one compared, one untimed and three timed
+    assert runs.count(True) == 4 * per_variant
+    assert runs.count(False) >= 4 * per_variant
