@@ -34,9 +34,10 @@ static bool fft_length_ok(int L) {
   }
 }
 
+// The passes of transform length L; setup_err null: without preparing their kernels on the device
 static bool pass_for_length(int L, PassLaunch* t, cudaError_t* setup_err) {
   switch (L) {
-#define LS_CASE(LL) case LL: *t = pass_table_##LL(); *setup_err = pass_setup_##LL(); return true;
+#define LS_CASE(LL) case LL: *t = pass_table_##LL(); if (setup_err) *setup_err = pass_setup_##LL(); return true;
     LS_CASE(16) LS_CASE(24) LS_CASE(32) LS_CASE(48) LS_CASE(64)
     LS_CASE(96) LS_CASE(128) LS_CASE(144) LS_CASE(192) LS_CASE(256) LS_CASE(288) LS_CASE(384)
 #undef LS_CASE
@@ -87,16 +88,30 @@ static int make_twiddles(int L, int R1, int R2, float2** tw, float2** tw2) {
   return LS_OK;
 }
 
+// The fused y/z pass of (ny, nz) (run == null: none)
+static YzLaunch yz_form(int ny, int nz) {
+  switch (ny) {
+#define LS_YZ_CASE(N) case N: return yz_row_##N(nz);
+    LS_YZ_LENGTHS(LS_YZ_CASE)
+#undef LS_YZ_CASE
+    default: return YzLaunch();
+  }
+}
+
+// Bytes of the Green values beside the octant: as the fused y/z pass reads them, and unfolded along x for the
+// dynamically scheduled z pass (0 where the grid has no such pass)
+static size_t gyz_bytes(const ls_grid& g) {
+  return yz_form(g.ny, g.nz).run ? (size_t)(g.nx + 1) * (g.ny + 1) * 2 * g.nz * sizeof(float2) : 0;
+}
+static size_t gxz_bytes(const ls_grid& g, const PassLaunch& pz) {
+  const bool has = pz.zdyn_ok && g.nz + 1 <= 256 && (2 * g.nx) % 16 == 0;
+  return has ? (size_t)2 * g.nx * (g.ny + 1) * (g.nz + 1) * sizeof(float2) : 0;
+}
+
 // Launcher, twiddle tables, column order and octant storage of the fused y/z pass, where (ny, nz) has
 // one; a failed allocation leaves the plan with the five passes.
 static int yz_setup(ls_plan* P) {
-  YzLaunch y;
-  switch (P->ny) {
-#define LS_YZ_CASE(N) case N: y = yz_row_##N(P->nz); break;
-    LS_YZ_LENGTHS(LS_YZ_CASE)
-#undef LS_YZ_CASE
-    default: break;
-  }
+  const YzLaunch y = yz_form(P->ny, P->nz);
   if (!y.run) return LS_OK;
   const double pi = 3.14159265358979323846;
   std::vector<float2> yt((size_t)2 * y.ra * y.csp, make_float2(0.f, 0.f)), zt((size_t)y.r1 * y.xr, make_float2(0.f, 0.f));
@@ -153,7 +168,7 @@ static int yz_setup(ls_plan* P) {
     return cudaMalloc(dst, bytes) == cudaSuccess && cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
   };
   const bool ok = y.setup() == cudaSuccess &&
-                  cudaMalloc((void**)&P->gyz, (size_t)(P->nx + 1) * (P->ny + 1) * 2 * P->nz * sizeof(float2)) == cudaSuccess &&
+                  cudaMalloc((void**)&P->gyz, gyz_bytes({P->nx, P->ny, P->nz})) == cudaSuccess &&
                   upload((void**)&P->yz_ytw, yt.data(), yt.size() * sizeof(float2)) &&
                   upload((void**)&P->yz_ztw, zt.data(), zt.size() * sizeof(float2)) &&
                   upload((void**)&P->yz_cols, cols.data(), cols.size() * sizeof(int));
@@ -1007,8 +1022,10 @@ size_t ls_workspace_bytes(const ls_grid* g, int n_views) {
   if (!g || n_views < 1) return 0;
   const size_t N = (size_t)g->nx * g->ny * g->nz;
   const size_t per_slot = (NVEC + 2 + 4) * N * sizeof(float2) + (size_t)g->nx * g->ny * sizeof(float2);
-  const size_t shared = (size_t)(g->nx + 1) * (g->ny + 1) * (g->nz + 1) * sizeof(float2) +
-                        (size_t)4 * N * sizeof(float2);
+  PassLaunch pz;
+  size_t shared = (size_t)(g->nx + 1) * (g->ny + 1) * (g->nz + 1) * sizeof(float2) + (size_t)4 * N * sizeof(float2) +
+                  gyz_bytes(*g);
+  if (pass_for_length(2 * g->nz, &pz, nullptr)) shared += gxz_bytes(*g, pz);
   return shared + per_slot * (size_t)n_views;
 }
 
@@ -1091,8 +1108,9 @@ int ls_plan_create(const ls_grid* grid, int padding, double k_b, double voxel, c
   }
   // the x-unfolded Green array of the dynamically scheduled z pass (where that pass exists); without
   // it the z pass runs in its other forms
-  if (rc == LS_OK && P->pz.zdyn_ok && P->nz + 1 <= 256 && (2 * P->nx) % 16 == 0) {
-    if (cudaMalloc(&P->gxz, (size_t)2 * P->nx * (P->ny + 1) * (P->nz + 1) * sizeof(float2)) != cudaSuccess) {
+  const size_t gxz = gxz_bytes({P->nx, P->ny, P->nz}, P->pz);
+  if (rc == LS_OK && gxz > 0) {
+    if (cudaMalloc(&P->gxz, gxz) != cudaSuccess) {
       cudaGetLastError();
       P->gxz = nullptr;
     }

@@ -70,8 +70,7 @@ constexpr int kChunkDefault = 2;   // BiCGStab iterations per round unless the o
 
 size_t plan_bytes(const ls_grid& g, int cap) {
   const size_t N = (size_t)g.nx * g.ny * g.nz;
-  return ls_workspace_bytes(&g, cap) + (size_t)cap * N * sizeof(float2) /* forward fields kept for gradients */ +
-         (size_t)4 * N * sizeof(float2) /* far-field kernels */;
+  return ls_workspace_bytes(&g, cap) + (size_t)cap * N * sizeof(float2) /* forward fields kept for gradients */;
 }
 
 }  // namespace
