@@ -805,6 +805,14 @@ int tune_forward(ls_plan* P, const float* f, int n, cudaStream_t st) {
   return engine_solve(P, n, st);
 }
 
+// Below this many voxels in flight (views times grid) the first iterations go out with the initial residual.  That
+// saves a wait for the host of 10 to 20 us in every solve, but costs one that starts converged (a warm start, a zero
+// potential) a chunk of launches in which every view is masked off.  us with the residual alone | with the
+// iterations: converged 32^3 x 1 84 | 113, 64^3 x 24 469 | 557, 192^3 x 1 489 | 599, x 2 843 | 1009, 128^3 x 60 5120 | 5409; not
+// converged 32^3 x 1 312 | 300, 64^3 x 24 2521 | 2510, 192^3 x 1 6215 | 6187.  From 2^22 on the wait is below half a
+// percent of the solve.
+constexpr size_t kSpeculateVoxels = (size_t)1 << 22;
+
 int engine_solve(ls_plan* P, int nslots, cudaStream_t st) {
   TraceRange range("solve");
   Engine& e = P->eng;
@@ -818,12 +826,11 @@ int engine_solve(ls_plan* P, int nslots, cudaStream_t st) {
   }
   const int chunk = P->opt.check_every > 0 ? P->opt.check_every : 2;
   // Rounds: a residual evaluation or a chunk of iterations.  The iterations that follow the initial
-  // residual need no look at the states in between (views that start converged are masked off), so the
-  // two go out together.
+  // residual need no look at the states in between (views that start converged are masked off).
   long long left = (long long)P->opt.max_iter * (P->opt.max_restarts + 2) / chunk + 16;
   if (P->inj_max_rounds >= 0) left = std::min(left, P->inj_max_rounds);
   int n_iter = 0, n_resid = nslots;
-  bool first = true;
+  bool first = (size_t)nslots * e.N < kSpeculateVoxels;
   if (left <= 0) LS_CUDA_TRY(cudaStreamSynchronize(st));   // slots_h is uploaded when this returns
   while (left > 0 && (n_iter > 0 || n_resid > 0)) {
     if (n_resid > 0) {
