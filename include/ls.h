@@ -382,13 +382,15 @@ enum ls_inject_kind {
                               /*   LS_ECUDA.  value = 0 turns it off                                         */
   LS_INJECT_BOUNDS_PROBE = 5  /* plan: value != 0: in the debug build (ls_debug_bounds) the plain first     */
                               /*   pass's slot check excludes the launch's last view, which then fails the   */
-                              /*   check (site 0x601) and is skipped; the normal build ignores it           */
+                              /*   check (site 0x601) and is skipped; 2: the fused y/z pass's check of its   */
+                              /*   output excludes a plane's last element (0x701), 3: the far field's inverse */
+                              /*   y pass's (0x803) its last one; the normal build ignores it                */
 };
 int ls_debug_inject(ls_plan* plan, int kind, long long value);
 
 /* Index checks of the debug build (the paper has no counterpart).  libls_debug.so is the library
  * compiled with LS_DEBUG_BOUNDS: its hot kernels (the five FFT passes, the bulk-staged first pass,
- * the z passes and the BiCGStab update) test every checked global or shared-memory index against
+ * the z passes, the fused y/z pass, the far field's inverse y pass and the BiCGStab update) test every checked global or shared-memory index against
  * the extents of its array; a failing check records a site code (kernel << 8 | access) and the
  * access is skipped, so a wrong index never faults.  *site (host, may be NULL) receives the first
  * recorded code over the library's translation units (0: none); clear = 1 resets the records.

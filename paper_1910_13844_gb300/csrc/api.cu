@@ -436,7 +436,7 @@ static void matvec_core(ls_plan* P, SlotSel sel, int nslots, const FxParams& fx_
   FxParams fx = fx_in;
   const bool fused = use_fused(P, nslots);
   fx.sel = counted(P, fx.sel, LS_K_FX);
-  fx.dbg_probe = P->inj_bounds_probe;
+  fx.dbg_probe = P->inj_bounds_probe == 1;
   fx.transposed = ix.transposed = fused ? 1 : 0;
   timed(P, LS_K_FX, nslots, st, [&] { P->px.fx(fx, nslots, st); });
   ix.sel = counted(P, sel, LS_K_IX);
@@ -456,6 +456,7 @@ static void matvec_core(ls_plan* P, SlotSel sel, int nslots, const FxParams& fx_
     yz.g = P->gyz;
     yz.ytw = P->yz_ytw; yz.ztw = P->yz_ztw; yz.cols = P->yz_cols;
     yz.sms = P->sms;
+    yz.dbg_probe = P->inj_bounds_probe == 2;
     timed_fused(P, nslots, st, [&] { P->yz.run(yz, nslots, st); });
     timed(P, LS_K_IX, nslots, st, [&] { P->px.ix(ix, nslots, st); });
     return;
@@ -611,6 +612,7 @@ static FarPassParams far_base(ls_plan* P, SlotSel sel, int nslots) {
   a.zchunks = (int)std::max(1LL, std::min((long long)P->nz / 8, (8LL * P->sms + ctas - 1) / ctas));
   a.k2 = P->k2hat;
   a.tw = P->tw_y;
+  a.dbg_probe = P->inj_bounds_probe == 3;
   return a;
 }
 
@@ -1711,7 +1713,7 @@ int ls_debug_inject(ls_plan* P, int kind, long long value) {
       return LS_OK;
     case LS_INJECT_BOUNDS_PROBE:
       if (!P) { set_last_error("null plan"); return LS_EINVAL; }
-      P->inj_bounds_probe = value != 0 ? 1 : 0;
+      P->inj_bounds_probe = value == 2 || value == 3 ? (int)value : value != 0 ? 1 : 0;
       return LS_OK;
     default:
       set_last_error("unknown injection kind %d", kind);

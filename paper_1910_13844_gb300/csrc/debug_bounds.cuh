@@ -28,6 +28,14 @@ enum BoundsSite : unsigned {
   BS_IX_PART = 0x403,     // IX: per-block partial sums
   BS_UPD_VEC = 0x501,     // update: vector element of a slot
   BS_UPD_PART = 0x502,    // update: per-block partial sums
+  BS_YZ_PLANE = 0x701,    // fused y/z pass: element of a plane of A1
+  BS_YZ_TILE = 0x702,     // fused y/z pass: entry of the tile in shared memory
+  BS_YZ_EXCH = 0x703,     // fused y/z pass: entry of a column's exchange area
+  BS_YZ_GREEN = 0x704,    // fused y/z pass: Green value
+  BS_FAR_SRC = 0x801,     // far field's inverse y pass: source element
+  BS_FAR_K2 = 0x802,      // far field's inverse y pass: element of a slice's kernel
+  BS_FAR_DST = 0x803,     // far field's inverse y pass: destination element
+  BS_FAR_SMEM = 0x804,    // far field's inverse y pass: exchange entry
   BS_SLOT = 0x601,        // any pass: slot index beyond the launch's slots
 };
 

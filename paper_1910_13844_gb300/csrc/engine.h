@@ -105,7 +105,8 @@ struct ls_plan {
   long long inj_max_rounds = -1;  // host rounds a solve may take (-1: the normal bound)
   int inj_z_stall = 0;            // the TMA-staged z pass waits on a barrier nothing completes
   long long inj_z_wait_ns = 0;    // per-view wait limit of the TMA-staged z pass (0: one second)
-  int inj_bounds_probe = 0;       // debug build: the first pass treats its last view as out of range
+  int inj_bounds_probe = 0;       // debug build: 1 the first pass treats its last view as out of range, 2 the fused y/z
+                                  // pass and 3 the far field's inverse y pass their last element
   // ls_matvec_noalloc: device address of the library's static scratch array on this plan's device,
   // looked up when the plan is created (null, with noalloc_rc set, if that failed)
   int device = 0;

@@ -68,6 +68,7 @@ struct FarPassParams {
   const float2* k2;            // K2hat [nz][2ny][2nx]
   const float2* tw;            // tw[j] = exp(-2 pi i j / L)
   int out_o, out_m;            // far_sum: cropped output window of y
+  int dbg_probe;               // debug build, test only: far_sum and far_iy take the last output element as out of range
 };
 
 struct ZParams {

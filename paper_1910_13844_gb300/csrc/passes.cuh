@@ -466,19 +466,26 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PS) k_far_iy(FarPassParams
 #pragma unroll
         for (int n1 = 0; n1 < R1; ++n1) {
           const size_t o = (size_t)(R2 * n1 + t) * a.ncont;
-          v[n1] = cmulc(src[o], __ldg(k + o));
+          if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, o + c, plane, a.src_stride), BS_FAR_SRC) &&
+              LS_IN_BOUNDS(z * plane + o + c < a.nz * plane, BS_FAR_K2))
+            v[n1] = cmulc(src[o], __ldg(k + o));
         }
       } else {
         for (int q = 0; q < a.zchunks; ++q) {
 #pragma unroll
-          for (int n1 = 0; n1 < R1; ++n1)
-            v[n1] = cadd(v[n1], src[q * plane + (size_t)(R2 * n1 + t) * a.ncont]);
+          for (int n1 = 0; n1 < R1; ++n1) {
+            const size_t o = q * plane + (size_t)(R2 * n1 + t) * a.ncont;
+            if (LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, o + c, a.zchunks * plane, a.src_stride), BS_FAR_SRC))
+              v[n1] = cadd(v[n1], src[o]);
+          }
         }
       }
     }
     Dft<R1, +1>::run(v);
 #pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) sm[(k1 * R2 + t) * P + p] = k1 ? cmulc(v[k1], __ldg(a.tw + k1 * t)) : v[0];
+    for (int k1 = 0; k1 < R1; ++k1)
+      if (LS_IN_BOUNDS((k1 * R2 + t) * P + p < L * P, BS_FAR_SMEM))
+        sm[(k1 * R2 + t) * P + p] = k1 ? cmulc(v[k1], __ldg(a.tw + k1 * t)) : v[0];
   }
   __syncthreads();
   if (c < a.ncont && t < R1) {
@@ -490,7 +497,11 @@ __global__ void __launch_bounds__(Geo<L>::T * Geo<L>::PS) k_far_iy(FarPassParams
 #pragma unroll
     for (int k2 = 0; k2 < R2 / 2; ++k2) {
       const int y = t + R1 * k2 - (ADJ ? 0 : a.out_o);
-      if (ADJ || (y >= 0 && y < a.out_m)) d[(size_t)y * a.ncont] = u[k2];
+      const size_t rows = ADJ ? (size_t)a.nz * (L / 2) : a.out_m;
+      if ((ADJ || (y >= 0 && y < a.out_m)) &&
+          LS_IN_BOUNDS(slot_elem_ok(slot, a.sel.nslots, ((ADJ ? (size_t)z * (L / 2) : 0) + y) * a.ncont + c,
+                                    rows * a.ncont - (a.dbg_probe ? 1 : 0), a.dst_stride), BS_FAR_DST))
+        d[(size_t)y * a.ncont] = u[k2];
     }
   }
 }
@@ -723,11 +734,15 @@ struct PassImpl {
   static dim3 far_grid(const FarPassParams& a, int nslots, int nz) {
     return dim3(nslots, (a.ncont + G::PS - 1) / G::PS, nz);
   }
-  static void far_sum(const FarPassParams& a, int nslots, cudaStream_t st) {
+  static void far_sum(const FarPassParams& a0, int nslots, cudaStream_t st) {
+    FarPassParams a = a0;
+    a.sel.nslots = nslots;
     launch_pdl((size_t)a.nz * (L / 2) * (a.ncont / 2), k_far_iy<L, false>, far_grid(a, nslots, 1), dim3(G::PS, G::T),
                G::smem_strided, st, a);
   }
-  static void far_iy(const FarPassParams& a, int nslots, cudaStream_t st) {
+  static void far_iy(const FarPassParams& a0, int nslots, cudaStream_t st) {
+    FarPassParams a = a0;
+    a.sel.nslots = nslots;
     launch_pdl((size_t)a.nz * (L / 2) * (a.ncont / 2), k_far_iy<L, true>, far_grid(a, nslots, a.nz), dim3(G::PS, G::T),
                G::smem_strided, st, a);
   }

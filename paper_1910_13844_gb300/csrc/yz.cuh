@@ -45,6 +45,7 @@ struct YzParams {
   const float2* ztw;             // [R1][R2+1]: exp(-2 pi i k1 n2 / (2 nz)) at [k1][n2]
   const int* cols;               // [2][ny/2][2]: tile position | j << 16 of the column pairs of parity P
   int sms;
+  int dbg_probe = 0;             // debug build, test only: a plane's last element is taken as out of range
 };
 
 // ny = RA RB on T threads per row.  RB = 2 T where it can be: a thread's loads are then pairs, and a row's are
@@ -347,19 +348,21 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
   auto load_rows = [&](const float2* plane, int g) {
     const int z = NZ % 16 == 0 ? row_a(g) : imin(row_a(g), NZ - 1);
     if constexpr (VEC) {
-      const float2* src = plane + z * NY + (SA * TY == RB ? 2 * ty : imin(2 * ty, RB - 2));
+      const int o = z * NY + (SA * TY == RB ? 2 * ty : imin(2 * ty, RB - 2));
 #pragma unroll
       for (int i = 0; i < RA; ++i) {
-        const float4 q = *reinterpret_cast<const float4*>(src + RB * i);
+        if (!LS_IN_BOUNDS(o + RB * i + 1 < NY * NZ, BS_YZ_PLANE)) continue;
+        const float4 q = *reinterpret_cast<const float4*>(plane + o + RB * i);
         v[0][i] = make_float2(q.x, q.y);
         v[SA - 1][i] = make_float2(q.z, q.w);
       }
     } else {
 #pragma unroll
       for (int s = 0; s < SA; ++s) {
-        const float2* src = plane + z * NY + (SA * TY == RB ? sub_a(s) : imin(sub_a(s), RB - 1));
+        const int o = z * NY + (SA * TY == RB ? sub_a(s) : imin(sub_a(s), RB - 1));
 #pragma unroll
-        for (int i = 0; i < RA; ++i) v[s][i] = src[RB * i];
+        for (int i = 0; i < RA; ++i)
+          if (LS_IN_BOUNDS(o + RB * i < NY * NZ, BS_YZ_PLANE)) v[s][i] = plane[o + RB * i];
       }
     }
   };
@@ -396,7 +399,7 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
             Dft<RA, -1>::run(v[s]);
             twiddle_out<RA, false, YT, false>(v[s], tq + W::TYA + (P * SA + s) * 2 * RA, yt + (mine ? b : 0), CSP, mine,
                                               [&](int c, float2 x) {
-              if (LS_IN_BOUNDS(z * PZ + c * CSP + b < NZ * PZ, BS_Z_SMEM)) row[c * CSP + b] = x;
+              if (LS_IN_BOUNDS(z * PZ + c * CSP + b < NZ * PZ, BS_YZ_TILE)) row[c * CSP + b] = x;
             });
           }
           if (g + NW < W::NRG) load_rows(plane, g + NW);
@@ -412,10 +415,12 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
               if (RA % TY == 0 || c < RA) {
                 float2 u[RB];
 #pragma unroll
-                for (int b = 0; b < RB; ++b) u[b] = row[c * CSP + b];
+                for (int b = 0; b < RB; ++b)
+                  if (LS_IN_BOUNDS(z * PZ + c * CSP + b < NZ * PZ, BS_YZ_TILE)) u[b] = row[c * CSP + b];
                 Dft<RB, -1>::run(u);
 #pragma unroll
-                for (int d = 0; d < RB; ++d) row[c * CSP + d] = u[d];
+                for (int d = 0; d < RB; ++d)
+                  if (LS_IN_BOUNDS(z * PZ + c * CSP + d < NZ * PZ, BS_YZ_TILE)) row[c * CSP + d] = u[d];
               }
             }
           }
@@ -442,7 +447,7 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
 #pragma unroll
             for (int s = 0; s < S2; ++s) {
               const int k1 = R1 % TZ == 0 ? tz + TZ * s : imin(tz + TZ * s, R1 - 1);
-              if (LS_IN_BOUNDS(ky >= 0 && ky < 2 * NY && k1 < R1, BS_Z_GREEN)) {
+              if (LS_IN_BOUNDS(ky >= 0 && ky < 2 * NY && k1 < R1, BS_YZ_GREEN)) {
 #pragma unroll
                 for (int h = 0; h < R2 / 2; ++h) {
                   const float4 x = __ldg(gc + h * R1 + k1);
@@ -459,10 +464,12 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
             const float2* src = col + (R2 % TZ == 0 ? n2 : imin(n2, R2 - 1)) * PZ;
             float2 v[R1];
 #pragma unroll
-            for (int n1 = 0; n1 < R1 / 2; ++n1) v[n1] = src[R2 * n1 * PZ];
+            for (int n1 = 0; n1 < R1 / 2; ++n1)
+              if (LS_IN_BOUNDS(src + R2 * n1 * PZ >= tile && src + R2 * n1 * PZ < tile + NZ * PZ, BS_YZ_TILE))
+                v[n1] = src[R2 * n1 * PZ];
             Dft<R1, -1, R1 / 2, R1>::run(v);
             twiddle_out<R1, false, ZT, true>(v, tq + W::TZ1 + s * 2 * R1, ztw + (mine ? n2 : 0), XR, mine, [&](int k1, float2 x) {
-              if (LS_IN_BOUNDS(k1 * XR + n2 < W::XP, BS_Z_SMEM)) xc[k1 * XR + n2] = x;
+              if (LS_IN_BOUNDS(k1 * XR + n2 < W::XP, BS_YZ_EXCH)) xc[k1 * XR + n2] = x;
             });
           }
           __syncwarp();
@@ -473,7 +480,8 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
             float2* ex = xc + (R1 % TZ == 0 ? k1 : imin(k1, R1 - 1)) * XR;
             float2 u[R2];
 #pragma unroll
-            for (int n2 = 0; n2 < R2; ++n2) u[n2] = ex[n2];
+            for (int n2 = 0; n2 < R2; ++n2)
+              if (LS_IN_BOUNDS(ex - xc + n2 < W::XP, BS_YZ_EXCH)) u[n2] = ex[n2];
             Dft<R2, -1>::run(u);
             if (adj) {
 #pragma unroll
@@ -485,7 +493,9 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
             Dft<R2, +1>::run(u);
             // in place: entry [k1][j1] is read by the thread of j1 in the last stage
             twiddle_out<R2, true, ZT, true>(u, tq + W::TZ2 + s * 2 * R2, ztw + (mine ? k1 : 0) * XR, 1, mine,
-                                            [&](int j1, float2 x) { ex[j1] = x; });
+                                            [&](int j1, float2 x) {
+              if (LS_IN_BOUNDS(ex - xc + j1 < W::XP, BS_YZ_EXCH)) ex[j1] = x;
+            });
           }
           __syncwarp();
           if (has) {
@@ -495,10 +505,12 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
               if (R2 % TZ == 0 || j1 < R2) {
                 float2 w[R1];
 #pragma unroll
-                for (int k1 = 0; k1 < R1; ++k1) w[k1] = xc[k1 * XR + j1];
+                for (int k1 = 0; k1 < R1; ++k1)
+                  if (LS_IN_BOUNDS(k1 * XR + j1 < W::XP, BS_YZ_EXCH)) w[k1] = xc[k1 * XR + j1];
                 Dft<R1, +1, R1, R1 / 2>::run(w);
 #pragma unroll
-                for (int j2 = 0; j2 < R1 / 2; ++j2) col[(j1 + R2 * j2) * PZ] = w[j2];
+                for (int j2 = 0; j2 < R1 / 2; ++j2)
+                  if (LS_IN_BOUNDS((pj & 0xffff) + (j1 + R2 * j2) * PZ < NZ * PZ, BS_YZ_TILE)) col[(j1 + R2 * j2) * PZ] = w[j2];
               }
             }
           }
@@ -524,10 +536,13 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
             float2* row = tile + z * PZ + c * CSP;
             float2 u[RB];
 #pragma unroll
-            for (int d = 0; d < RB; ++d) u[d] = row[d];
+            for (int d = 0; d < RB; ++d)
+              if (LS_IN_BOUNDS(z * PZ + c * CSP + d < NZ * PZ, BS_YZ_TILE)) u[d] = row[d];
             Dft<RB, +1>::run(u);
             twiddle_out<RB, true, YT, false>(u, tq + W::TYB + (P * SB + s) * 2 * RB, yt + c * CSP, 1, mine,
-                                             [&](int b, float2 x) { row[b] = x; });
+                                             [&](int b, float2 x) {
+              if (LS_IN_BOUNDS(z * PZ + c * CSP + b < NZ * PZ, BS_YZ_TILE)) row[b] = x;
+            });
           }
         }
         __syncwarp();
@@ -540,7 +555,8 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
           for (int s = 0; s < SA; ++s) {
             const int b = SA * TY == RB ? sub_a(s) : imin(sub_a(s), RB - 1);
 #pragma unroll
-            for (int c = 0; c < RA; ++c) o[s][c] = row[c * CSP + b];
+            for (int c = 0; c < RA; ++c)
+              if (LS_IN_BOUNDS(z * PZ + c * CSP + b < NZ * PZ, BS_YZ_TILE)) o[s][c] = row[c * CSP + b];
             Dft<RA, +1>::run(o[s]);
             if (P) twist<RA, +1>(o[s]);
             // tensor-memory accesses are warp-collective: every lane takes part, with its own values
@@ -561,15 +577,18 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
             if (has && (RB % (2 * TY) == 0 || sub_a(0) < RB)) {
 #pragma unroll
               for (int i = 0; i < RA; ++i)
-                *reinterpret_cast<float4*>(plane + z * NY + RB * i + sub_a(0)) =
-                    make_float4(o[0][i].x, o[0][i].y, o[SA - 1][i].x, o[SA - 1][i].y);
+                if (LS_IN_BOUNDS(z * NY + RB * i + sub_a(0) + 1 < NY * NZ - (a.dbg_probe ? 1 : 0), BS_YZ_PLANE))
+                  *reinterpret_cast<float4*>(plane + z * NY + RB * i + sub_a(0)) =
+                      make_float4(o[0][i].x, o[0][i].y, o[SA - 1][i].x, o[SA - 1][i].y);
             }
           } else {
 #pragma unroll
             for (int s = 0; s < SA; ++s)
               if (has && (RB % TY == 0 || sub_a(s) < RB)) {
 #pragma unroll
-                for (int i = 0; i < RA; ++i) plane[z * NY + RB * i + sub_a(s)] = o[s][i];
+                for (int i = 0; i < RA; ++i)
+                  if (LS_IN_BOUNDS(z * NY + RB * i + sub_a(s) < NY * NZ - (a.dbg_probe ? 1 : 0), BS_YZ_PLANE))
+                    plane[z * NY + RB * i + sub_a(s)] = o[s][i];
               }
           }
         }
