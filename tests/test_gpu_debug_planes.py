@@ -87,3 +87,47 @@ def run_debug_child(code, **env):
 @pytest.mark.gpu
 def test_checks_pass_and_are_made():
     run_debug_child(CHILD)
+
+
+FORMS = PREAMBLE + r'''
+name = torch.cuda.get_device_name().replace(" ", "_")
+
+def case(shape, views, line):
+    nz, ny, nx = shape
+    open(os.environ["LS_AUTOTUNE_CACHE"], "w").write(f"{name}:{nx}x{ny}x{nz}:{views} {line}\n")
+    f64 = potential(ph.random_ellipsoids(shape, count=3, rmin=2, rmax=6, dn_max=0.04, seed=3))
+    f = to_dev(torch, f64, torch.float32)
+    kvec = ph.cone_directions(views, 0.8) * KB
+    plan = ls.Plan(shape, KB, H, tol=1e-6)
+    assert plan.autotune(views, f)["from_cache"] == 1
+    u, far, code, stats = plan.forward(f, plan.plane_waves(kvec))
+    g, gcode, _ = plan.gradient(f, far.clone(), u_fwd=u)
+    torch.cuda.synchronize()
+    assert code == ls.LS_OK and gcode == ls.LS_OK, (shape, line, stats)
+    assert site() == 0, (shape, line)
+    op = model.Operator(model.setup_from_optics(shape, LAM, ETA_B, H))
+    for q in range(views):
+        u_o = model.forward(op, f64, model.plane_wave(shape, H, kvec[q]), tol=1e-12)
+        assert rel(u[q].cpu().numpy(), u_o) < 1e-4, (shape, line)
+        assert rel(far[q].cpu().numpy(), op.farfield_fft(f64 * u_o)) < 1e-4, (shape, line)
+    assert bool(torch.isfinite(g).all())
+    plan.close()
+
+# z_tma ix_prefetch fx_views_fastest check_every use_graphs ms ms z_split strided_wide views_per_launch z_persist fx_bulk fused
+# the three passes at the lengths whose z pass has a kernel or a split of its own (144: column groups; 128, 192 and 384:
+# several stage-2 sub-transforms per thread), in every form, and at one that does not
+for shape in [(72, 16, 16), (64, 16, 16), (96, 16, 16), (192, 16, 16), (24, 16, 32)]:
+    for form in ["1 1 0 2 1 1 1 0 0 0 0 0 0", "1 0 1 2 0 1 1 1 1 1 1 0 0", "1 1 0 4 1 1 1 0 1 0 2 1 0", "0 1 0 2 1 1 1 0 0 0 0 0 0"]:
+        case(shape, 2, form)
+    print(shape, "ok", flush=True)
+# the fused pass beside every form of the first and last pass
+for form in ["1 1 1 2 1 1 1 0 0 0 0 0 1", "1 0 0 2 1 1 1 0 0 0 0 1 1", "1 1 0 4 0 1 1 0 0 1 0 1 1", "1 0 1 8 1 1 1 0 0 2 0 0 1"]:
+    for shape in [(32, 32, 32), (24, 16, 96), (72, 72, 16)]:
+        case(shape, 3, form)
+print("all ok", flush=True)
+'''
+
+
+@pytest.mark.gpu
+def test_every_form_of_a_tuned_plan(tmp_path):
+    run_debug_child(FORMS, LS_AUTOTUNE_CACHE=str(tmp_path / "tune.txt"))

@@ -2,7 +2,11 @@
 the ranges of FY, Z and IY inside one another, the three passes one after the other."""
 import pytest
 
-from gpu_common import torch_and_lib
+import phantoms as ph
+from oracle import model
+
+from gpu_common import ETA_B, H, KB, LAM, potential, rel, to_dev, torch_and_lib
+from test_gpu_autotune import VARIANTS
 from test_trace import _run
 
 SOLVE = """
@@ -50,7 +54,7 @@ def solve_forms(tmp_path, monkeypatch, shape, views, line):
     lines = _run(tmp_path, SOLVE.format(shape=shape, views=views, line=line, cache=tmp_path / "tune.txt"))
     # the far field that follows the solve runs FY alone
     n = len(forms(lines)) - 1
-    assert n > 4
+    assert n >= 4
     return forms(lines)[:n]
 
 
@@ -88,3 +92,42 @@ def test_the_tuner_tries_the_first_and_last_pass_in_both_forms(tmp_path):
     per_variant = 1 + 4   # one compared, one untimed and three timed
     assert runs.count(True) == 4 * per_variant
     assert runs.count(False) >= 4 * per_variant
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fused", [0, 1])
+@pytest.mark.parametrize("variant", VARIANTS)
+def test_every_variant_in_both_forms(tmp_path, monkeypatch, variant, fused):
+    # SOLVE compares the fields with the oracle's
+    torch_and_lib()
+    v = [str(x) for x in variant]
+    line = " ".join(v[:5]) + " 1.0 1.0 " + " ".join(v[5:]) + f" {fused}"
+    assert set(solve_forms(tmp_path, monkeypatch, (32, 32, 32), 3, line)) == {bool(fused)}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(72, 72, 16), (144, 144, 16), (8, 64, 32), (48, 8, 96)])
+def test_several_planes_per_cta_where_the_fused_pass_is_a_choice(tmp_path, monkeypatch, shape):
+    torch, ls = torch_and_lib()
+    views, (nz, ny, nx) = 70, shape
+    cache = tmp_path / "tune.txt"
+    name = torch.cuda.get_device_name().replace(" ", "_")
+    cache.write_text(f"{name}:{nx}x{ny}x{nz}:{views} 1 1 0 2 1 1.0 1.0 0 0 0 0 0 1\n")
+    monkeypatch.setenv("LS_AUTOTUNE_CACHE", str(cache))
+    f = to_dev(torch, potential(ph.random_potential_like(shape, seed=4)), torch.float32)
+    op = model.Operator(model.setup_from_optics(shape, LAM, ETA_B, H))
+    plan = ls.Plan(shape, KB, H)
+    assert plan.autotune(views, f)["from_cache"] == 1
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.view_as_complex(torch.randn((views,) + shape + (2,), device="cuda", generator=g))
+    y = torch.empty_like(x)
+    ls.ls_profile(plan.handle, True)
+    ls.ls_matvec_batch(plan.handle, f, x, y, True)
+    torch.cuda.synchronize()
+    times = ls.ls_profile(plan.handle, False)
+    # one launch stands for the three passes: its time is divided between them 1 : 2 : 1
+    assert times["fy"][0] > 0 and times["fy"][0] == times["iy"][0] == pytest.approx(times["z"][0] / 2, rel=1e-6)
+    for q in (0, 1, 33, 69):
+        ref = op.A(x[q].cpu().numpy().astype("complex128"), f.cpu().numpy().astype("float64"), True)
+        assert rel(y[q].cpu().numpy(), ref) < 3e-6, q
+    plan.close()
