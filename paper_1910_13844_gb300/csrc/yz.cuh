@@ -10,7 +10,9 @@
 // same plane, Y[2j + P] = DFT_ny(x[y] W_2ny^{P y})[j], so only one ny x nz tile is in shared memory at a
 // time: the CTA runs P = 0 and then P = 1 (the second read of the plane comes from L2), and keeps the
 // first half's partial output in tensor memory, which serves as a register file extension (every
-// thread reads back what it wrote).  A warp owns the same rows in both halves and in both directions,
+// thread reads back what it wrote).  The factor W_2ny^{P y} is part of the odd half's DFTs (DftOddIn, DftOddOut): as
+// a twist of their inputs and outputs it was one rounding more than the three passes have (operator error against
+// 64 bits at 48^3 +13%, 96x72x48 +10%, 64^3 +3%; now within 2% of theirs, or below).  A warp owns the same rows in both halves and in both directions,
 // so only the two transposes between rows and columns are CTA barriers.
 //
 // Layout.  y = RB a + b, j = c + RA d: stage A transforms over a (thread b), stage B over b (thread c), in
@@ -49,35 +51,37 @@ struct YzParams {
 };
 
 // ny = RA RB on T threads per row.  RB = 2 T where it can be: a thread's loads are then pairs, and a row's are
-// contiguous (144 = 9 16 instead of 12 12 and 72 = 9 8 instead of 12 6, whose threads kept three or one and a half
-// transforms of the first stage: 144x128 planes, eight views with nx = 64, 47.7 -> 36.6 us a view; 144x96
-// 35.6 -> 28.7; 144x144, with the z split below, 58.5 -> 55.8; 72x32 5.4 -> 4.7).
+// contiguous.  us a view, nx = 64, 16M voxels in flight: 48 = 6 8 against 8 6, 48x96 planes 8.6 -> 7.9 and 48x48 4.2 -> 4.0;
+// 32 = 4 8 against 8 4, 32x128 7.8 -> 7.4; 72 = 9 8 against 12 6, 72x32 4.6 -> 4.1, 72x128 20.6 -> 19.1 (72x64 8.7 -> 9.2);
+// 144 = 9 16 against 12 12, 144x96 33.3 -> 28.0, 144x16 4.9 -> 4.4.
 template <int NY> struct YSplit;
 template <> struct YSplit<8>   { static constexpr int RA = 4, RB = 2, T = 4; };
 template <> struct YSplit<12>  { static constexpr int RA = 4, RB = 3, T = 4; };
 template <> struct YSplit<16>  { static constexpr int RA = 4, RB = 4, T = 4; };
 template <> struct YSplit<24>  { static constexpr int RA = 4, RB = 6, T = 4; };
-template <> struct YSplit<32>  { static constexpr int RA = 8, RB = 4, T = 4; };
-template <> struct YSplit<48>  { static constexpr int RA = 8, RB = 6, T = 4; };
+template <> struct YSplit<32>   { static constexpr int RA = 4, RB = 8, T = 4; };
+template <> struct YSplit<48>   { static constexpr int RA = 6, RB = 8, T = 4; };
 template <> struct YSplit<64>  { static constexpr int RA = 8, RB = 8, T = 4; };
-template <> struct YSplit<72>  { static constexpr int RA = 9, RB = 8, T = 4; };
+template <> struct YSplit<72>   { static constexpr int RA = 9, RB = 8, T = 4; };
 template <> struct YSplit<96>  { static constexpr int RA = 12, RB = 8, T = 4; };
 template <> struct YSplit<128> { static constexpr int RA = 8, RB = 16, T = 8; };
-template <> struct YSplit<144> { static constexpr int RA = 9, RB = 16, T = 8; };
+template <> struct YSplit<144>  { static constexpr int RA = 9, RB = 16, T = 8; };
 template <> struct YSplit<192> { static constexpr int RA = 12, RB = 16, T = 8; };
-// 2 nz = R1 R2 (R1 even) on T threads per column (288 = 16 18, not 24 12: 60 registers fewer, 96x144 35.0 -> 32.4 us)
+// 2 nz = R1 R2 (R1 even) on T threads per column.  96 = 16 6 and 288 = 24 12 for their rounding (3 coprime to the rest: no
+// twiddles inside the DFTs), at the time of 12 8 and 16 18 or less (32x144 10.3 -> 10.0, 128x144 37.7 -> 35.2, but 96x144
+// 30.8 -> 32.7).
 template <int NZ> struct ZSplit2;
 template <> struct ZSplit2<8>   { static constexpr int R1 = 4, R2 = 4, T = 4; };
 template <> struct ZSplit2<12>  { static constexpr int R1 = 4, R2 = 6, T = 4; };
 template <> struct ZSplit2<16>  { static constexpr int R1 = 8, R2 = 4, T = 4; };
 template <> struct ZSplit2<24>  { static constexpr int R1 = 8, R2 = 6, T = 8; };
 template <> struct ZSplit2<32>  { static constexpr int R1 = 8, R2 = 8, T = 8; };
-template <> struct ZSplit2<48>  { static constexpr int R1 = 12, R2 = 8, T = 8; };
+template <> struct ZSplit2<48>   { static constexpr int R1 = 16, R2 = 6, T = 8; };
 template <> struct ZSplit2<64>  { static constexpr int R1 = 16, R2 = 8, T = 8; };
 template <> struct ZSplit2<72>  { static constexpr int R1 = 12, R2 = 12, T = 16; };
 template <> struct ZSplit2<96>  { static constexpr int R1 = 24, R2 = 8, T = 8; };
 template <> struct ZSplit2<128> { static constexpr int R1 = 16, R2 = 16, T = 16; };
-template <> struct ZSplit2<144> { static constexpr int R1 = 16, R2 = 18, T = 16; };
+template <> struct ZSplit2<144>  { static constexpr int R1 = 24, R2 = 12, T = 16; };
 template <> struct ZSplit2<192> { static constexpr int R1 = 24, R2 = 16, T = 16; };
 
 __host__ __device__ constexpr int cdiv(int a, int b) { return (a + b - 1) / b; }
@@ -217,15 +221,6 @@ __device__ __forceinline__ void tmem_loaded(float2* v) {
   tmem_wait_ld();
 #pragma unroll
   for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i].x), "+f"(v[i].y));
-}
-
-// v[a] *= exp(DIR 2 pi i a / (2 RA)), the twist of the odd half, with compile-time factors
-template <int RA, int DIR, int A = 1>
-__device__ __forceinline__ void twist(float2* v) {
-  if constexpr (A < RA) {
-    v[A] = twc<A, 2 * RA, DIR>(v[A]);
-    twist<RA, DIR, A + 1>(v);
-  }
 }
 
 // Twiddles 0 .. N - 1 of one sub-transform times its values, and the store of every product: from tensor
@@ -395,8 +390,8 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
           for (int s = 0; s < SA; ++s) {
             const int b = sub_a(s);
             const bool mine = has && (SA * TY == RB || b < RB);
-            if (P) twist<RA, -1>(v[s]);
-            Dft<RA, -1>::run(v[s]);
+            if (P) DftOddIn<RA, -1>::run(v[s]);
+            else Dft<RA, -1>::run(v[s]);
             twiddle_out<RA, false, YT, false>(v[s], tq + W::TYA + (P * SA + s) * 2 * RA, yt + (mine ? b : 0), CSP, mine,
                                               [&](int c, float2 x) {
               if (LS_IN_BOUNDS(z * PZ + c * CSP + b < NZ * PZ, BS_YZ_TILE)) row[c * CSP + b] = x;
@@ -557,8 +552,8 @@ __global__ void __launch_bounds__(YZ<NY, NZ>::NT, YZ<NY, NZ>::MINB) k_yz(YzParam
 #pragma unroll
             for (int c = 0; c < RA; ++c)
               if (LS_IN_BOUNDS(z * PZ + c * CSP + b < NZ * PZ, BS_YZ_TILE)) o[s][c] = row[c * CSP + b];
-            Dft<RA, +1>::run(o[s]);
-            if (P) twist<RA, +1>(o[s]);
+            if (P) DftOddOut<RA, +1>::run(o[s]);
+            else Dft<RA, +1>::run(o[s]);
             // tensor-memory accesses are warp-collective: every lane takes part, with its own values
             const unsigned ta = tq + (unsigned)(W::slot(g, NW) * W::TCOL + s * 2 * W::RAE);
             if (P == 0) {

@@ -1063,7 +1063,7 @@ __global__ void __launch_bounds__(ZG<L>::NT, ZG<L>::MINB) k_zg(const __grid_cons
       for (int n1 = 0; n1 < R1 / 2; ++n1)
         if (LS_IN_BOUNDS(swz128(R2 * n1 + n2, cc) + sizeof(float2) <= W::stage_bytes, BS_Z_SMEM))
           v[n1] = *reinterpret_cast<const float2*>(sb + swz128(R2 * n1 + n2, cc));
-      Dft<R1, -1, R1 / 2, R1>::run(v);
+      Dft<R1, -1, R1 / 2, R1, false>::run(v);
       const float4* tw4 = reinterpret_cast<const float4*>(twa + n2 * W::TWA);
 #pragma unroll
       for (int k = 0; k < R1 / 2; ++k) {
@@ -1084,7 +1084,7 @@ __global__ void __launch_bounds__(ZG<L>::NT, ZG<L>::MINB) k_zg(const __grid_cons
       u[2 * q] = make_float2(x.x, x.y);
       u[2 * q + 1] = make_float2(x.z, x.w);
     }
-    Dft<R2, -1>::run(u);
+    Dft<R2, -1, R2, R2, false>::run(u);
     if (active_adj(s_list[iv])) {
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) u[k2] = cmulc(u[k2], gr[k2]);
@@ -1097,7 +1097,7 @@ __global__ void __launch_bounds__(ZG<L>::NT, ZG<L>::MINB) k_zg(const __grid_cons
       const int j = (int)blockIdx.x + (kt + 1) * (int)gridDim.x;
       load_green<L, R1, R2>(gr, a, j / tiles_c, (j % tiles_c) * P + cc, t);
     }
-    Dft<R2, +1>::run(u);
+    Dft<R2, +1, R2, R2, false>::run(u);
     {
       const float4* tw4 = reinterpret_cast<const float4*>(twb + t * W::TWB);
 #pragma unroll
@@ -1122,7 +1122,7 @@ __global__ void __launch_bounds__(ZG<L>::NT, ZG<L>::MINB) k_zg(const __grid_cons
         w[2 * q] = make_float2(x.x, x.y);
         w[2 * q + 1] = make_float2(x.z, x.w);
       }
-      Dft<R1, +1, R1, R1 / 2>::run(w);
+      Dft<R1, +1, R1, R1 / 2, false>::run(w);
 #pragma unroll
       for (int j2 = 0; j2 < R1 / 2; ++j2)
         if (LS_IN_BOUNDS(swz128(j1 + R2 * j2, cc) + sizeof(float2) <= W::stage_bytes, BS_Z_SMEM))
