@@ -377,8 +377,8 @@ def run_gpu(args):
     barrier()
     ms_e2e = e0.elapsed_time(e1)
 
-    # the five passes once more with every view active (ls_matvec_batch), for per-pass GB/s free of
-    # the masked launches of converged views
+    # the operator's passes once more with every view active (ls_matvec_batch), for per-pass GB/s free
+    # of the masked launches of converged views
     ls.ls_matvec_batch(plan.handle, f0, uin, u)
     torch.cuda.synchronize()
     ls.ls_profile(plan.handle, True)

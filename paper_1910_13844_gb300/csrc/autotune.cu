@@ -268,8 +268,8 @@ extern "C" int ls_autotune(ls_plan* P, int n_views, const float* f, ls_tune* out
   double sv_ms = -1.0;
   {
     // the fused y/z pass in place of the three (tuned) passes, where the grid has it: before the launch
-    // structure, whose best differs (60 views at 128^3: 30 a launch with three passes, whose intermediates are
-    // larger, all 60 with one; the choice made for three passes cost a solve with one 3%)
+    // structure, whose costs differ (solve of 60 views at 128^3 with all, 30, 15 and 8 a launch: three passes 59.7,
+    // 59.8, 61.7, 63.8 ms, one 53.9, 54.5, 56.2, 58.1)
     if (form[1].ms > 0) {
       const double three = time_ms(st, kSolveReps, solve);
       set_form(1);

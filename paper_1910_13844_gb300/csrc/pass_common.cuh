@@ -204,8 +204,9 @@ __host__ __device__ constexpr int rows_per_cta(int t) {
 // Threads per row and rows per CTA of the plain first pass.  One thread per sub-transform of the longer stage;
 // for 128 = 16 8 of the shorter one (eight threads that make two 8-point transforms each), since half of 16 would
 // have nothing to load: the pass in 64^3 x 24 operators 2.02 -> 1.64 us a view (60 views 1.82 -> 1.40), with 16 rows a
-// CTA; with 32 it was slower in the iteration's modes.  The other unequal splits idle less, and their CTAs with
-// twice the rows were 5-10% slower.
+// CTA; with 32 it was slower in the iteration's modes.  32 = 8 4 idles as many threads, but nx = 16 makes grids bound by
+// their launches and keeps the general form.  The other unequal splits idle less, and their CTAs with twice the rows
+// were 5-10% slower.
 template <int L>
 struct FxRows {
   static constexpr int T = imax(Radix<L>::R1, Radix<L>::R2), P = rows_per_cta(T);
