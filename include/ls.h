@@ -192,7 +192,8 @@ int ls_matvec_noalloc(const ls_plan* plan, const float* f, const ls_c64* x, ls_c
  * The kernels read and write these vectors where they are; vectors that overlap one
  * another (u_out[q] == u_in[q]) go through the workspace.
  * Returns LS_OK, LS_NOT_CONVERGED, LS_BREAKDOWN or LS_TIMEOUT (worst view), or an error;
- * LS_ECUDA also when a z-pass wait on its own TMA copy gave up (bounded, one second). */
+ * LS_ECUDA also when a z-pass wait on its own TMA copy gave up (bounded, one second).  After an
+ * error that arose while the solve ran, u_out and far hold no result (u_out may have been written). */
 int ls_forward(ls_plan* plan, const float* f, int n_views, const ls_c64* const* u_in,
                ls_c64* const* u_out, ls_c64* const* far, ls_stats* stats, void* cuda_stream);
 

@@ -25,9 +25,9 @@
 // read from tensor memory; a thread transforms the columns ky and -ky one after the other with the same
 // Green values in registers; the plane and the Green values are read with 16-byte loads.
 //
-// Measured, us a view against FY, Z and IY as three launches: 128^3 x 60 views 57.0 -> 50.6 (16 views under ncu:
-// FMA pipe 59% and shared-memory pipe 65% of their peaks, 78 MB of DRAM traffic a view where the three passes
-// move 340), 64^3 x 24 9.4 -> 6.4, 96^3 x 16 28.9 -> 23.7, 144^3 x 1 198 -> 137.  The FP32 instructions alone are
+// Measured, us a view against FY, Z and IY as three launches: 128^3 x 60 views 57.0 -> 51.1 (16 views under ncu:
+// FMA pipe 58% and shared-memory pipe 64% of their peaks, 80 MB of DRAM traffic a view where the three passes
+// move 340), 64^3 x 24 9.4 -> 6.3, 96^3 x 16 28.9 -> 23.3, 144^3 x 1 198 -> 135.  The FP32 instructions alone are
 // 29 us a view at 128^3; the rest is the two pipes taking turns between the barriers.
 #pragma once
 
