@@ -159,10 +159,11 @@ struct YZ {
   // (at 128 a thread they would spill: 57 instead of 52 us a view at 128^3)
   static constexpr bool CROSS = 65536 / (NT * MINB) >= 160;
   // Against FY, Z and IY as three launches, measured over all pairs of lengths with nx = 64: one view, 1.1 to
-  // 2.2 times as fast wherever the tile fits; 16M voxels in flight, 1.0 to 1.5 times, but 0.86 to 0.98 of
-  // their rate with ny = 72 and nz = 72, 128 and more, with ny = 144 and nz = 72 or 144 (a quarter to a half of
-  // the lanes idle in one of their stages, eight or nine warps an SM), with nz = 8 and with ny = 8 and nz >= 48
-  // (few warps).
+  // 2.2 times as fast wherever the tile fits; 16M voxels in flight, 1.0 to 1.5 times (24x72 and 24x192 0.93 and 0.97),
+  // but 0.85 to 0.92 of their rate with ny = 72 and nz = 128 and more (72x72 1.01), 0.91 and 0.98 with ny = 144 and
+  // nz = 144 and 72 (a quarter to a half of the lanes idle in one of their stages, eight or nine warps an SM), 0.79 to
+  // 1.05 with nz = 8, and 0.65 to 0.71 with ny = 8 and nz = 48 and 64 (few warps; 1.1 to 1.5 from nz = 72 on, where the
+  // line could move).
   static constexpr bool large_ok = !(NY == 72 && NZ >= 72 && NZ != 96) && !(NY == 144 && (NZ == 72 || NZ == 144)) &&
                                    NZ != 8 && !(NY == 8 && NZ >= 48);
   static constexpr size_t smem_z = tile_bytes + col_bytes + (size_t)NW * warp_bytes;
